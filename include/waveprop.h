@@ -28,6 +28,12 @@
  *     every source/receiver must lie inside the computational grid,
  *     [-nbl h, (n-1+nbl) h] on each axis (PROP_EINVAL otherwise; y = 0 for
  *     PROP_ELASTIC2D, which has no absorbing cells in y).
+ *   - The stencil passes are TMA-fed where the rows of a field are whole
+ *     16-byte units.  Other computational nz get rows padded by up to three
+ *     floats inside the library (state access keeps packed rows); rows shorter
+ *     than 8 floats per float of padding, grids that the padding would take to
+ *     2^32 elements, staggered-pair TTI handles and elastic or acoustic handles
+ *     with 16-bit checkpoints keep packed rows and run the pipelined passes.
  *   - Buffers may be host or device pointers (detected per pointer with
  *     cudaPointerGetAttributes).  The caller owns every buffer passed in or
  *     out; the library owns the handle and all device memory it allocates,
@@ -177,7 +183,8 @@ int prop_gradient(prop_t *p, const float *wavelet, const float *src_xyz, int nsr
  * the first derivatives of zeta and of the forward field; needs 6 more
  * scratch fields than prop_gradient.
  * Any computational nz with the centred operators (TMA-fed passes when nz +
- * 2 nbl is a multiple of 4, the pipelined passes otherwise).
+ * 2 nbl is a multiple of 4; otherwise the pipelined passes, whose rounding the
+ * strongly cancelling tilt and azimuth gradients show).
  * PROP_EINVAL for a non-TTI handle, or for tti_operator = 1 with a
  * computational nz that is not a multiple of 4 (its half-point imaging runs
  * on the TMA-fed passes, which need 16-byte rows). */
@@ -200,8 +207,8 @@ int prop_backward(prop_t *p, const float *resid, float *grad, float *src_grad);
  * shot i computes exactly prop_forward(shots[i], wavelet[i], src_xyz[i],
  * nsrc[i], rec_xyz[i], nrec[i], traces[i]) -- bitwise the same traces.
  * When every shot is TTI with the centred operators (or every shot is
- * elastic), with the same space order and nt, a computational nz that is a
- * multiple of 4 and windows of at most 16 M computational points on
+ * elastic), with the same space order and nt, on the TMA-fed passes and
+ * windows of at most 16 M computational points on
  * average (WAVEPROP_LOCKSTEP=1: any size, =0: never), each time step is
  * one launch of each pass over a table of all the shots' tiles (each shot
  * keeping its own model window, grid and x-extent) beside the shots'
@@ -233,7 +240,7 @@ int prop_forward_batch(prop_t *const *shots, int nshots, const float *const *wav
  * handle keeps its own message); the other shots still run.  Each shot's
  * work arrays are released after its gradient (prop_trim), so later waves
  * can use that memory; its wavefield state then reads as zero.
- * TTI shots of a wave (centred operators, computational nz a multiple of 4)
+ * TTI shots of a wave (centred operators, on the TMA-fed passes)
  * share their step launches: the k-th step of every such shot runs as one
  * launch of each pass over a table of all the shots' tiles (set
  * WAVEPROP_BATCH_LAUNCH=0 to launch shot by shot).  A wave whose shots are

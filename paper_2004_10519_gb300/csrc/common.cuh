@@ -6,7 +6,7 @@
 
 WP_DEV long long gidx(const GridDev &g, int x, int y, int z)
 {
-    return ((long long)x * g.NY + y) * g.NZ + z;
+    return ((long long)x * g.NY + y) * g.PZ + z;
 }
 
 // depth (cells, continuous) of coordinate s into the absorbing layer of an

@@ -203,15 +203,16 @@ el_grad_b_kernel(GridDev g, FDW w, Fields9 s, Fields9 xf0, float *__restrict__ f
 // update v^{k+1} = g (v^k + (dt/h) b_avg Dtau(tau^k)) gives
 // (dt/h) Dtau(tau^k) = (v^{k+1}/g - v^k) / b_avg at each velocity point, so
 // fp_c = vbar_c (v^{k+1}_c / g_c - v^k_c) / b_avg,c equals the product of
-// el_grad_b_kernel.  Two z points per thread, 8-byte accesses (NZ even, as
-// on the TMA path that uses it); tapers and averages as in the TMA passes.
+// el_grad_b_kernel.  Two z points per thread, 8-byte accesses (rows of an
+// even pitch, as on the TMA path that uses it; beyond an odd NZ the pitch holds
+// zero wavefields and the model's edge values); tapers and averages as in the TMA passes.
 __global__ void __launch_bounds__(256)
 el_face2_kernel(GridDev g, Fields9 s, Fields9 xf0, Fields9 xf1, const float *__restrict__ bu,
                 float *__restrict__ f0, float *__restrict__ f1, float *__restrict__ f2)
 {
     const int x = blockIdx.z, y = blockIdx.y * 8 + threadIdx.y, z = 2 * (blockIdx.x * 32 + threadIdx.x);
     if (y >= g.NY || z >= g.NZ) return;
-    const long long pl = (long long)g.NY * g.NZ, q = ((long long)x * g.NY + y) * g.NZ + z;
+    const long long pl = (long long)g.NY * g.PZ, q = gidx(g, x, y, z);
     auto ld = [](const float *p, long long o) { return __ldg(reinterpret_cast<const float2 *>(p + o)); };
     // accumulate into the face-product sums (read before written, own points only)
     auto st = [](float *p, long long o, float a, float b) {
@@ -220,13 +221,14 @@ el_face2_kernel(GridDev g, Fields9 s, Fields9 xf0, Fields9 xf1, const float *__r
         *d = make_float2(v.x + a, v.y + b);
     };
     const float2 b0 = ld(bu, q);
-    const float2 bX = x + 1 < g.NX ? ld(bu, q + pl) : b0, bY = y + 1 < g.NY ? ld(bu, q + g.NZ) : b0;
+    const float2 bX = x + 1 < g.NX ? ld(bu, q + pl) : b0, bY = y + 1 < g.NY ? ld(bu, q + g.PZ) : b0;
     const float bz2 = z + 2 < g.NZ ? __ldg(bu + q + 2) : b0.y;
     const float *tz = g.tab + 2 * (g.NX + g.NY);
     const float gxn = __ldg(g.tab + 2 * x), gxh = __ldg(g.tab + 2 * x + 1);
     const float gyn = __ldg(g.tab + 2 * g.NX + 2 * y), gyh = __ldg(g.tab + 2 * g.NX + 2 * y + 1);
     const float gzn0 = __ldg(tz + 2 * z), gzh0 = __ldg(tz + 2 * z + 1);
-    const float gzn1 = __ldg(tz + 2 * z + 2), gzh1 = __ldg(tz + 2 * z + 3);
+    const int z1 = min(z + 1, g.NZ - 1);
+    const float gzn1 = __ldg(tz + 2 * z1), gzh1 = __ldg(tz + 2 * z1 + 1);
     const float2 u0 = ld(s.f[0], q), u1 = ld(s.f[1], q), u2 = ld(s.f[2], q);
     const float2 a0 = ld(xf0.f[0], q), a1 = ld(xf0.f[1], q), a2 = ld(xf0.f[2], q);
     const float2 c0 = ld(xf1.f[0], q), c1 = ld(xf1.f[1], q), c2 = ld(xf1.f[2], q);
@@ -325,9 +327,9 @@ WP_DEV float adj_sedge(const GridDev &g, const float *tc, const float *__restric
 {
     if (!(x >= 0 && x < g.NX && y >= 0 && y < g.NY && z >= 0 && z < g.NZ)) return 0.f;
     const long long q = gidx(g, x, y, z);
-    const long long d1 = A1 == 0 ? (x + 1 < g.NX ? (long long)g.NY * g.NZ : 0)
-                                 : (y + 1 < g.NY ? (long long)g.NZ : 0);
-    const long long d2 = A2 == 1 ? (y + 1 < g.NY ? (long long)g.NZ : 0) : (z + 1 < g.NZ ? 1 : 0);
+    const long long d1 = A1 == 0 ? (x + 1 < g.NX ? (long long)g.NY * g.PZ : 0)
+                                 : (y + 1 < g.NY ? (long long)g.PZ : 0);
+    const long long d2 = A2 == 1 ? (y + 1 < g.NY ? (long long)g.PZ : 0) : (z + 1 < g.NZ ? 1 : 0);
     const float mavg = 0.25f * (__ldg(mu + q) + __ldg(mu + q + d1) + __ldg(mu + q + d2) +
                                 __ldg(mu + q + d1 + d2));
     const float gt = tp(g, x, A1 == 0, y, (A1 == 1) || (A2 == 1), z, A2 == 2);
@@ -340,8 +342,8 @@ WP_DEV float adj_bv(const GridDev &g, const float *__restrict__ v, const float *
     if (!(x >= 0 && x < g.NX && y >= 0 && y < g.NY && z >= 0 && z < g.NZ)) return 0.f;
     const long long q = gidx(g, x, y, z);
     long long d = 0;
-    if (c == 0) d = x + 1 < g.NX ? (long long)g.NY * g.NZ : 0;
-    else if (c == 1) d = y + 1 < g.NY ? (long long)g.NZ : 0;
+    if (c == 0) d = x + 1 < g.NX ? (long long)g.NY * g.PZ : 0;
+    else if (c == 1) d = y + 1 < g.NY ? (long long)g.PZ : 0;
     else d = z + 1 < g.NZ ? 1 : 0;
     return 0.5f * (__ldg(bu + q) + __ldg(bu + q + d)) * v[q];
 }

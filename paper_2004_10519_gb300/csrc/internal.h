@@ -14,12 +14,13 @@
 
 #define WP_MAXM 8   // space order up to 16
 
-// Computational grid as seen by the kernels.  Index (x,y,z) -> (x*NY + y)*NZ + z.
+// Computational grid as seen by the kernels.  Index (x,y,z) -> (x*NY + y)*PZ + z.
 struct GridDev {
     int NX, NY, NZ;          // computational grid
+    int PZ;                  // row pitch in floats (>= NZ): a multiple of 4 where the TMA-fed passes run
     int nbl, px, py, pz;     // absorbing width, physical grid
     int nby;                 // absorbing width on the y faces (0 in 2D)
-    long long N;             // NX*NY*NZ
+    long long N;             // elements of a field, NX*NY*PZ
     float h, ih, dt;         // spacing, 1/h, time step
     float sig0;              // TTI damping: sigma(d) = sig0 * (d/L)^2 per axis [1/s]
     float cer;               // elastic Cerjan coefficient per cell (0.015)
@@ -76,6 +77,7 @@ struct prop_s {
     float *tab = nullptr;    // per-axis absorbing-layer tables (GridDev::tab)
     int xchunk = 8;          // planes per CTA of the x-streaming stencil kernels
     int tile_y = 16;         // rows (y) per tile of the TMA-fed passes: 8, 16 or 32
+    bool pipelined = false;  // keep this handle (or call) on the pipelined passes (row_pitch, prop_gradient_aniso)
     // saved forward run for prop_backward
     bool saved = false;
     bool aniso = false;      // TTI gradient also w.r.t. eps, delta (prop_gradient_aniso)
@@ -151,7 +153,8 @@ int el_launch_fast(prop_s *P, float *const *S, float dt_sign);
 // one 2D elastic step of S = (vx, vz, txx, tzz, txz); dt_sign = -1: the
 // transposed step in the adjoint-modelling variables
 int el2_launch(prop_s *P, float *const *S, float dt_sign);
-// TMA-fed passes (stencil_tma.cu): usable when NZ % 4 == 0
+// TMA-fed passes (stencil_tma.cu): usable when the row pitch is a multiple of 4
+// and the handle is not held on the pipelined passes (P->pipelined)
 bool tma_usable(const prop_s *P);
 // acoustic step (S[0] = u^n, S[1] = u^{n-1} <- u^{n+1}); grad != NULL:
 // transposed step with imaging grad -= dt^2 uf (L lam) / m
@@ -270,13 +273,14 @@ void k_set_int(prop_s *P, int *p, int v);
 // mode 0: coef = scale; mode 1: coef = scale / A (TTI, A = m(1+sig dt/2));
 // mode 2: coef = scale (3 lambda + 2 mu) (elastic adjoint in s = C tbar);
 // mode 3: as mode 1 into f0 = lam_p, and (1 + 2 eps), sqrt(1 + 2 delta) times
-// that into f1 = zeta_p, f2 = zeta_r (TTI transposed step, zeta = C lam);
+// that into f1 = zeta_p, f2 = zeta_r (TTI transposed step, zeta = C lam; with
+// lr = lam_r, zeta is formed from the new lam instead, as the pipelined passes do);
 // grad_u != NULL: grad[cell] -= u[cell] * scale*sum / m  (TTI imaging of the
 // residual injection)
 // (tdev != NULL: t read from device memory)
 void sp_inject(prop_s *P, const SparseDev *S, const float *traces, int nt, int t, float scale,
                int mode, float *f0, float *f1, float *f2, const float *grad_u, float *grad,
-               const int *tdev = nullptr);
+               const int *tdev = nullptr, const float *lr = nullptr);
 // as sp_record but each field sum is divided by (3 lambda + 2 mu) at the cell
 // (trace of tbar from s = C tbar)
 void sp_record_trace_s(prop_s *P, const SparseDev *S, const float *f0, const float *f1,

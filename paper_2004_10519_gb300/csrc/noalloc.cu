@@ -153,7 +153,8 @@ int run(prop_s *P, const prop_desc *d, const float *const *model, const float *w
     GridDev &g = P->g;
     g.nbl = d->nbl; g.nby = d->nbl; g.px = d->nx; g.py = d->ny; g.pz = d->nz;
     g.NX = d->nx + 2 * d->nbl; g.NY = d->ny + 2 * d->nbl; g.NZ = d->nz + 2 * d->nbl;
-    g.N = (long long)g.NX * g.NY * g.NZ;
+    g.PZ = g.NZ;
+    g.N = (long long)g.NX * g.NY * g.PZ;
     g.h = d->h; g.ih = 1.f / d->h; g.cer = 0.015f;
     if (!fd_weights(P->M, P->w.c, P->w.b)) return wp_fail(P, PROP_EINVAL, "FD weights");
     const size_t np = (size_t)d->nx * d->ny * d->nz, N = (size_t)g.N;

@@ -45,7 +45,7 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
                               int t, float scale, int mode, const float *__restrict__ m,
                               const float *__restrict__ lam, const float *__restrict__ mu,
                               float *f0, float *f1, float *f2, const float *__restrict__ gu,
-                              float *grad, const int *__restrict__ tdev)
+                              float *grad, const int *__restrict__ tdev, const float *__restrict__ lr)
 {
     // lam, mu: the elastic Lame parameters; for TTI (mode 3) epsilon, delta
     int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -56,13 +56,13 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
     const long long q = cell[j];
     float coef = scale;
     if (mode == 1 || mode == 3) {
-        const int z = (int)(q % g.NZ), y = (int)((q / g.NZ) % g.NY), x = (int)(q / ((long long)g.NZ * g.NY));
+        const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY), x = (int)(q / ((long long)g.PZ * g.NY));
         const float A = m[q] * (1.f + 0.5f * tti_sigma(g, x, y, z) * g.dt);
         coef = scale / A;
     } else if (mode == 2 || mode == 4) {
         // residual into u = g C tbar: g (3 lambda + 2 mu) on each diagonal
         // component (mode 4, the x-z plane: g (2 lambda + 2 mu) on xx, zz)
-        const int z = (int)(q % g.NZ), y = (int)((q / g.NZ) % g.NY), x = (int)(q / ((long long)g.NZ * g.NY));
+        const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY), x = (int)(q / ((long long)g.PZ * g.NY));
         const float gn = g.tab[2 * x] * g.tab[2 * g.NX + 2 * y] * g.tab[2 * (g.NX + g.NY) + 2 * z];
         coef = scale * ((mode == 2 ? 3.f : 2.f) * lam[q] + 2.f * mu[q]) * gn;
     }
@@ -71,8 +71,9 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
     if (mode == 3) {
         // TTI transposed step: the residual enters lam_p; keep zeta = C lam
         // (f1, f2) consistent: zeta_p += (1 + 2 eps) v, zeta_r += sqrt(1 + 2 delta) v
-        f1[q] += (1.f + 2.f * lam[q]) * v;
-        f2[q] += sqrtf(1.f + 2.f * mu[q]) * v;
+        const float c1 = 1.f + 2.f * lam[q], c2 = sqrtf(1.f + 2.f * mu[q]);
+        f1[q] = lr ? c1 * f0[q] + c2 * lr[q] : f1[q] + c1 * v;
+        f2[q] = lr ? c2 * f0[q] + lr[q] : f2[q] + c2 * v;
     } else {
         if (f1) f1[q] += v;
         if (f2) f2[q] += v;
@@ -95,8 +96,8 @@ __global__ void record_s_kernel(GridDev g, int n, const long long *__restrict__ 
         const float wc = w[8 * i + c];
         if (wc != 0.f) {
             // tr(tbar) = tr(u) / (g (3 lambda + 2 mu)) at a node
-            const int z = (int)(q % g.NZ), y = (int)((q / g.NZ) % g.NY),
-                      x = (int)(q / ((long long)g.NZ * g.NY));
+            const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY),
+                      x = (int)(q / ((long long)g.PZ * g.NY));
             const float gn = g.tab[2 * x] * g.tab[2 * g.NX + 2 * y] * g.tab[2 * (g.NX + g.NY) + 2 * z];
             s += wc * (f0[q] + f1[q] + (f2 ? f2[q] : 0.f)) / ((nl * lam[q] + 2.f * mu[q]) * gn);
         }
@@ -125,7 +126,7 @@ __global__ void extend_kernel(GridDev g, const float *__restrict__ phys, float *
 {
     long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (q >= g.N) return;
-    const int z = (int)(q % g.NZ), y = (int)((q / g.NZ) % g.NY), x = (int)(q / ((long long)g.NZ * g.NY));
+    const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY), x = (int)(q / ((long long)g.PZ * g.NY));
     const int i = clampi(x - g.nbl, 0, g.px - 1), j = clampi(y - g.nby, 0, g.py - 1),
               k = clampi(z - g.nbl, 0, g.pz - 1);
     const float v = phys[((long long)i * g.py + j) * g.pz + k];
@@ -168,8 +169,9 @@ __global__ void normals_kernel(long long n, const float *th, const float *ph, fl
 // computational cells c + nbl, plus the whole layer in front of c = 0 and
 // behind c = n - 1.  Folding the three axes in turn is the transpose of the
 // three-axis extension, with at most nbl + 1 terms per output.
+// (rows of `in` are `pitch` elements apart, those of `out` are packed)
 __global__ void fold_axis_kernel(const float *__restrict__ in, float *__restrict__ out, int d0, int d1,
-                                 int d2, int axis, int n, int nbl)
+                                 int d2, int pitch, int axis, int n, int nbl)
 {
     const int o0 = axis == 0 ? n : d0, o1 = axis == 1 ? n : d1, o2 = axis == 2 ? n : d2;
     const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -177,8 +179,8 @@ __global__ void fold_axis_kernel(const float *__restrict__ in, float *__restrict
     const int k = (int)(q % o2), j = (int)((q / o2) % o1), i = (int)(q / ((long long)o2 * o1));
     const int c = axis == 0 ? i : (axis == 1 ? j : k), N = axis == 0 ? d0 : (axis == 1 ? d1 : d2);
     const int lo = c == 0 ? 0 : c + nbl, hi = c == n - 1 ? N - 1 : c + nbl;
-    const long long st = axis == 0 ? (long long)d1 * d2 : (axis == 1 ? (long long)d2 : 1LL);
-    const long long base = ((long long)(axis == 0 ? 0 : i) * d1 + (axis == 1 ? 0 : j)) * d2 + (axis == 2 ? 0 : k);
+    const long long st = axis == 0 ? (long long)d1 * pitch : (axis == 1 ? (long long)pitch : 1LL);
+    const long long base = ((long long)(axis == 0 ? 0 : i) * d1 + (axis == 1 ? 0 : j)) * pitch + (axis == 2 ? 0 : k);
     float s = 0.f;
     for (int t = lo; t <= hi; t++) s += in[base + t * st];
     out[q] = s;
@@ -327,7 +329,7 @@ int sp_host_tables(prop_s *P, const float *xyz, int n, const int *trace_of_point
                 for (int d = 0; d < 2; d++, c++) {
                     const double wt = (a ? f[0] : 1 - f[0]) * (b ? f[1] : 1 - f[1]) * (d ? f[2] : 1 - f[2]);
                     if (wt == 0.0) continue;
-                    const long long q = ((long long)(i0[0] + a) * g.NY + (i0[1] + b)) * g.NZ + (i0[2] + d);
+                    const long long q = ((long long)(i0[0] + a) * g.NY + (i0[1] + b)) * g.PZ + (i0[2] + d);
                     T.ridx[8 * (size_t)i + c] = q;
                     T.rw[8 * (size_t)i + c] = (float)wt;
                     ent.emplace_back(q, trace_of_point ? trace_of_point[i] : i, (float)wt);
@@ -415,14 +417,15 @@ void k_set_int(prop_s *P, int *p, int v)
 }
 
 void sp_inject(prop_s *P, const SparseDev *S, const float *traces, int nt, int t, float scale,
-               int mode, float *f0, float *f1, float *f2, const float *grad_u, float *grad, const int *tdev)
+               int mode, float *f0, float *f1, float *f2, const float *grad_u, float *grad, const int *tdev,
+               const float *lr)
 {
     if (S->ncell <= 0) return;
     inject_kernel<<<nblk(S->ncell), NB, 0, P->stream>>>(P->g, S->ncell, S->cell, S->cell_ptr,
                                                         S->ent_trace, S->ent_w, traces, nt, t, scale,
                                                         mode, P->m, mode == 3 ? P->eps : P->lam,
                                                         mode == 3 ? P->del : P->mu, f0, f1, f2,
-                                                        grad_u, grad, tdev);
+                                                        grad_u, grad, tdev, lr);
     P->kern_launches++;
 }
 
@@ -462,9 +465,9 @@ void k_fold(prop_s *P, const float *comp, float *phys, float *s1, float *s2)
     const GridDev &g = P->g;
     const long long n1 = (long long)g.NX * g.NY * g.pz, n2 = (long long)g.NX * g.py * g.pz,
                     n3 = (long long)g.px * g.py * g.pz;
-    fold_axis_kernel<<<nblk(n1), NB, 0, P->stream>>>(comp, s1, g.NX, g.NY, g.NZ, 2, g.pz, g.nbl);
-    fold_axis_kernel<<<nblk(n2), NB, 0, P->stream>>>(s1, s2, g.NX, g.NY, g.pz, 1, g.py, g.nby);
-    fold_axis_kernel<<<nblk(n3), NB, 0, P->stream>>>(s2, phys, g.NX, g.py, g.pz, 0, g.px, g.nbl);
+    fold_axis_kernel<<<nblk(n1), NB, 0, P->stream>>>(comp, s1, g.NX, g.NY, g.NZ, g.PZ, 2, g.pz, g.nbl);
+    fold_axis_kernel<<<nblk(n2), NB, 0, P->stream>>>(s1, s2, g.NX, g.NY, g.pz, g.pz, 1, g.py, g.nby);
+    fold_axis_kernel<<<nblk(n3), NB, 0, P->stream>>>(s2, phys, g.NX, g.py, g.pz, g.pz, 0, g.px, g.nbl);
     P->kern_launches += 3;
 }
 

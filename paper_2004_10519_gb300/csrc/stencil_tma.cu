@@ -17,6 +17,10 @@
 // 32 x 32 tile, two rows per thread).
 // z-derivatives read a window of M+1 float2 per field; x-derivatives use
 // per-thread float2 register queues.
+// Rows are a pitch of a multiple of 4 floats apart (16-byte rows for TMA), at
+// least NZ.  The maps end at NZ, so the padding reads as zero; where NZ is odd
+// the second point of a row's last pair is padding, and what the passes write
+// there is zero (`two` below; without it where the zero inputs already give it).
 // Offsets are 32-bit (the runtime keeps N below 2^32).  Every mbarrier wait
 // is bounded in time: on expiry the warp sets bit 2 of the error word and
 // leaves, the producer first waiting (again bounded) for its copies in
@@ -57,7 +61,7 @@ struct VMaps {
 // shared-memory offsets and the y/z Cerjan factors of its two z points.
 template <int M>
 struct ElCtx {
-    bool act;
+    bool act, two;           // two: the second point is in the grid, not row padding
     unsigned q0;             // in-plane offset of the first point
     int cy, cz, c2, ii;      // rows/columns in the halo boxes and the interior box
     int yb1, zb2;            // +1 box row of y+1 and column of z+2 (clamped at the grid end)
@@ -70,7 +74,8 @@ WP_DEV ElCtx<M> el_ctx(const GridDev &g, int z0, int y0, int tz, int ty)
     ElCtx<M> t;
     const int z = z0 + 2 * tz, y = y0 + ty;
     t.act = y < g.NY && z < g.NZ;
-    t.q0 = t.act ? (unsigned)y * g.NZ + z : 0u;
+    t.two = z + 1 < g.NZ;
+    t.q0 = t.act ? (unsigned)y * g.PZ + z : 0u;
     const float *tabz = g.tab + 2 * (g.NX + g.NY);
     const int zc0 = min(z, g.NZ - 1), zc1 = min(z + 1, g.NZ - 1), yc = min(y, g.NY - 1);
     t.gzn0 = __ldg(tabz + 2 * zc0);
@@ -131,7 +136,7 @@ template <int M>
 WP_DEV void v_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, float2 (&qxx)[2 * M],
                       float2 (&qxy)[2 * M], float2 (&qxz)[2 * M])
 {
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
     const float2 Z2 = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < 2 * M - 1; j++) {
@@ -186,11 +191,11 @@ WP_DEV void v_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
         const float2 bY = lds2(sb + t.yb1 * B::PC + c2);
         const float bz2 = sb[ty * B::PC + t.zb2];
         const float gxn = __ldg(g.tab + 2 * x), gxh = __ldg(g.tab + 2 * x + 1);
-        const unsigned q = x * (unsigned)g.NY * (unsigned)g.NZ + t.q0;
+        const unsigned q = x * (unsigned)g.NY * (unsigned)g.PZ + t.q0;
         // face averages of buoyancy and tapers at the three velocity points
         const float bxa = 0.5f * (b0.x + bxn.x), bxb = 0.5f * (b0.y + bxn.y);
         const float bya = 0.5f * (b0.x + bY.x), byb = 0.5f * (b0.y + bY.y);
-        const float bza = 0.5f * (b0.x + b0.y), bzb = 0.5f * (b0.y + bz2);
+        const float bza = 0.5f * (b0.x + (t.two ? b0.y : b0.x)), bzb = 0.5f * (b0.y + bz2);
         const float gx0 = gxh * t.gyn * t.gzn0, gx1 = gxh * t.gyn * t.gzn1;
         const float gy0 = gxn * t.gyh * t.gzn0, gy1 = gxn * t.gyh * t.gzn1;
         const float gz0 = gxn * t.gyn * t.gzh0, gz1 = gxn * t.gyn * t.gzh1;
@@ -199,9 +204,9 @@ WP_DEV void v_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
             st2(s.f[1], q, gy0 * (v1.x + c * bya * d1a), gy1 * (v1.y + c * byb * d1b));
             st2(s.f[2], q, gz0 * (v2.x + c * bza * d2a), gz1 * (v2.y + c * bzb * d2b));
         } else {
-            const float u0a = gx0 * (v0.x - c * d0a), u0b = gx1 * (v0.y - c * d0b);
-            const float u1a = gy0 * (v1.x - c * d1a), u1b = gy1 * (v1.y - c * d1b);
-            const float u2a = gz0 * (v2.x - c * d2a), u2b = gz1 * (v2.y - c * d2b);
+            const float u0a = gx0 * (v0.x - c * d0a), u0b = t.two ? gx1 * (v0.y - c * d0b) : 0.f;
+            const float u1a = gy0 * (v1.x - c * d1a), u1b = t.two ? gy1 * (v1.y - c * d1b) : 0.f;
+            const float u2a = gz0 * (v2.x - c * d2a), u2b = t.two ? gz1 * (v2.y - c * d2b) : 0.f;
             st2(s.f[0], q, u0a, u0b);
             st2(s.f[1], q, u1a, u1b);
             st2(s.f[2], q, u2a, u2b);
@@ -321,7 +326,7 @@ template <int M>
 WP_DEV void t_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, float2 (&qvx)[2 * M],
                       float2 (&qvy)[2 * M], float2 (&qvz)[2 * M])
 {
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
     const float2 Z2 = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < 2 * M - 1; j++) {
@@ -373,7 +378,7 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
         const float *T = S + L::OT + ii;
         const float2 t0 = lds2(T), t1 = lds2(T + IS), t2 = lds2(T + 2 * IS);
         const float2 t3 = lds2(T + 3 * IS), t4 = lds2(T + 4 * IS), t5 = lds2(T + 5 * IS);
-        const unsigned q = x * (unsigned)g.NY * (unsigned)g.NZ + t.q0;
+        const unsigned q = x * (unsigned)g.NY * (unsigned)g.PZ + t.q0;
         if (MODE == 0) {
             const float *R0 = S + L::OM0, *R1 = S + L::OM1;
             const float2 m0 = lds2(R0 + ty * B::PC + c2), my = lds2(R0 + t.yb1 * B::PC + c2);
@@ -384,10 +389,12 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
             const float gyn = t.gyn, gyh = t.gyh, gzn0 = t.gzn0, gzn1 = t.gzn1, gzh0 = t.gzh0, gzh1 = t.gzh1;
             const float gn0 = gxn * gyn * gzn0, gn1 = gxn * gyn * gzn1;
             // averages of mu over the 4 nodes around each edge (the pair's
-            // second lane is the first point's z+1 neighbour)
+            // second lane is the first point's z+1 neighbour, which is clamped
+            // to the point itself at the last node)
             const float mxya = 0.25f * (m0.x + mx.x + my.x + mxy_.x);
-            const float mxza = 0.25f * (m0.x + mx.x + m0.y + mx.y);
-            const float myza = 0.25f * (m0.x + my.x + m0.y + my.y);
+            const float m0n = t.two ? m0.y : m0.x, mxn = t.two ? mx.y : mx.x, myn = t.two ? my.y : my.x;
+            const float mxza = 0.25f * (m0.x + mx.x + m0n + mxn);
+            const float myza = 0.25f * (m0.x + my.x + m0n + myn);
             const float mxyb = 0.25f * (m0.y + mx.y + my.y + mxy_.y);
             const float mxzb = 0.25f * (m0.y + mx.y + m0z + mxz);
             const float myzb = 0.25f * (m0.y + my.y + m0z + myz);
@@ -400,12 +407,12 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
             st2(s.f[7], q, gxh * gyn * gzh0 * (t4.x + c * mxza * gxza), gxh * gyn * gzh1 * (t4.y + c * mxzb * gxzb));
             st2(s.f[8], q, gxn * gyh * gzh0 * (t5.x + c * myza * gyza), gxn * gyh * gzh1 * (t5.y + c * myzb * gyzb));
         } else if (MODE == 1) {
-            st2(s.f[3], q, t0.x - c * exa, t0.y - c * exb);
-            st2(s.f[4], q, t1.x - c * eya, t1.y - c * eyb);
-            st2(s.f[5], q, t2.x - c * eza, t2.y - c * ezb);
-            st2(s.f[6], q, t3.x - c * gxya, t3.y - c * gxyb);
-            st2(s.f[7], q, t4.x - c * gxza, t4.y - c * gxzb);
-            st2(s.f[8], q, t5.x - c * gyza, t5.y - c * gyzb);
+            st2(s.f[3], q, t0.x - c * exa, t.two ? t0.y - c * exb : 0.f);
+            st2(s.f[4], q, t1.x - c * eya, t.two ? t1.y - c * eyb : 0.f);
+            st2(s.f[5], q, t2.x - c * eza, t.two ? t2.y - c * ezb : 0.f);
+            st2(s.f[6], q, t3.x - c * gxya, t.two ? t3.y - c * gxyb : 0.f);
+            st2(s.f[7], q, t4.x - c * gxza, t.two ? t4.y - c * gxzb : 0.f);
+            st2(s.f[8], q, t5.x - c * gyza, t.two ? t5.y - c * gyzb : 0.f);
         } else {
             const float2 gl = lds2(S + L::OG + ii), gm = lds2(S + L::OG + IS + ii);
             st2(o.f[0], q, gl.x + c * (t0.x + t1.x + t2.x) * (exa + eya + eza),
@@ -569,8 +576,8 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
         return;
     }
     const bool act = y < g.NY && z < g.NZ;
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
-    const unsigned q0 = act ? (unsigned)y * g.NZ + z : 0u;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
+    const unsigned q0 = act ? (unsigned)y * g.PZ + z : 0u;
     const float2 Z2 = make_float2(0.f, 0.f);
     float2 qp[Q], qr[Q];
 #pragma unroll
@@ -765,8 +772,8 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
         return;
     }
     const bool act = y < g.NY && z < g.NZ;
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
-    const unsigned q0 = act ? (unsigned)y * g.NZ + z : 0u;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
+    const unsigned q0 = act ? (unsigned)y * g.PZ + z : 0u;
     const float2 Z2 = make_float2(0.f, 0.f);
     float2 qe[Q], qf[Q];
 #pragma unroll
@@ -779,7 +786,8 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
     const float *sx = g.tab, *sy = g.tab + g.NX, *sz = g.tab + g.NX + g.NY;
     const float dt2 = g.dt * g.dt, hdt = 0.5f * g.dt;
     const float syv = act ? __ldg(sy + y) : 0.f;
-    const float syz0 = act ? syv + __ldg(sz + z) : 0.f, syz1 = act ? syv + __ldg(sz + z + 1) : 0.f;
+    const float syz0 = act ? syv + __ldg(sz + z) : 0.f, syz1 = act ? syv + __ldg(sz + min(z + 1, g.NZ - 1)) : 0.f;
+    const bool two = z + 1 < g.NZ, padded = g.PZ != g.NZ;
     const int c2 = 2 * tz, ii = ty * FZ + c2;
     const int iy = (ty + M) * B::YC + c2, izr = ty * B::ZC, cz = B::MZ + c2;
     for (int x = xa; x < xb; x++) {
@@ -821,8 +829,9 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
                 const float2 p0 = lds2(I + L::PP * IS), r0 = lds2(I + L::RP * IS);
                 const float2 e_ = lds2(I + L::EP * IS), d_ = lds2(I + L::DE * IS);
                 const float sxv = __ldg(sx + x);
-                const float h0[2] = {h0a * g.ih, h0b * g.ih}, hz[2] = {hza * g.ih, hzb * g.ih};
-                const float M2[2] = {mm.x, mm.y}, E2[2] = {e_.x, e_.y}, D2[2] = {d_.x, d_.y};
+                const float h0[2] = {__fmul_rn(h0a, g.ih), __fmul_rn(h0b, g.ih)};
+                const float hz[2] = {__fmul_rn(hza, g.ih), __fmul_rn(hzb, g.ih)};
+                const float M2[2] = {mm.x, two ? mm.y : mm.x}, E2[2] = {e_.x, e_.y}, D2[2] = {d_.x, d_.y};
                 const float P1[2] = {p1.x, p1.y}, R1[2] = {r1.x, r1.y}, P0[2] = {p0.x, p0.y}, R0[2] = {r0.x, r0.y};
                 const float SYZ[2] = {syz0, syz1};
                 float pn[2], rn[2], Lp[2], Lr[2], c1[2], c2[2];
@@ -831,17 +840,29 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
                     c1[i] = 1.f + 2.f * E2[i];
                     c2[i] = sqrtf(1.f + 2.f * D2[i]);
                     if (!ADJ) {
-                        Lp[i] = c1[i] * h0[i] + c2[i] * hz[i];
-                        Lr[i] = c2[i] * h0[i] + hz[i];
+                        Lp[i] = __fmaf_rn(c1[i], h0[i], __fmul_rn(c2[i], hz[i]));
+                        Lr[i] = __fmaf_rn(c2[i], h0[i], hz[i]);
                     } else {
                         Lp[i] = h0[i];
                         Lr[i] = hz[i];
                     }
-                    const float sd = hdt * (sxv + SYZ[i]);
-                    const float A = M2[i] * (1.f + sd), Bc = M2[i] * (1.f - sd);
-                    pn[i] = (dt2 * Lp[i] + 2.f * M2[i] * P1[i] - Bc * P0[i]) / A;
-                    rn[i] = (dt2 * Lr[i] + 2.f * M2[i] * R1[i] - Bc * R0[i]) / A;
+                    const float sig = __fadd_rn(sxv, SYZ[i]);
+                    const float A = __fmul_rn(M2[i], __fmaf_rn(hdt, sig, 1.f)),
+                                Bc = __fmul_rn(M2[i], __fmaf_rn(-hdt, sig, 1.f));
+                    // (dt^2 L + 2 m u) - B u-: of the first sum one product is
+                    // rounded and the other fused, which one is the only thing in
+                    // which the pipelined passes differ; padded rows follow them
+                    // (the operations of a point are spelt out here, so that the
+                    // rounding is not the compiler's choice)
+                    const float m2 = 2.f * M2[i];
+                    const float tp = padded ? __fmaf_rn(m2, P1[i], __fmul_rn(dt2, Lp[i]))
+                                            : __fmaf_rn(dt2, Lp[i], __fmul_rn(m2, P1[i]));
+                    const float tr = padded ? __fmaf_rn(m2, R1[i], __fmul_rn(dt2, Lr[i]))
+                                            : __fmaf_rn(dt2, Lr[i], __fmul_rn(m2, R1[i]));
+                    pn[i] = __fmaf_rn(-Bc, P0[i], tp) / A;
+                    rn[i] = __fmaf_rn(-Bc, R0[i], tr) / A;
                 }
+                if (!two) pn[1] = rn[1] = 0.f;
                 st2(pp, q, pn[0], pn[1]);
                 st2(rp, q, rn[0], rn[1]);
                 if (ADJ) {
@@ -990,8 +1011,8 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
         return;
     }
     const bool a0 = ya < g.NY && z < g.NZ, a1 = a0 && ya + 1 < g.NY;
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
-    const unsigned qa = a0 ? (unsigned)ya * g.NZ + z : 0u, qb = a1 ? qa + g.NZ : 0u;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
+    const unsigned qa = a0 ? (unsigned)ya * g.PZ + z : 0u, qb = a1 ? qa + g.PZ : 0u;
     const float2 Z2 = make_float2(0.f, 0.f);
     float2 qu0[Q], qu1[Q];
 #pragma unroll
@@ -1002,7 +1023,7 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
         qu1[j] = a1 && in ? ldg2(u1, xq * pl + qb) : Z2;
     }
     const float *sx = g.tab, *sy = g.tab + g.NX, *sz = g.tab + g.NX + g.NY;
-    const float sz0 = a0 ? __ldg(sz + z) : 0.f, sz1 = a0 ? __ldg(sz + z + 1) : 0.f;
+    const float sz0 = a0 ? __ldg(sz + z) : 0.f, sz1 = a0 ? __ldg(sz + min(z + 1, g.NZ - 1)) : 0.f;
     const float sy0 = a0 ? __ldg(sy + ya) : 0.f, sy1 = a1 ? __ldg(sy + ya + 1) : 0.f;
     const float2 syz[2] = {make_float2(sy0 + sz0, sy0 + sz1), make_float2(sy1 + sz0, sy1 + sz1)};
     const float hdt = 0.5f * g.dt;
@@ -1455,11 +1476,11 @@ int acu_launch_tma(prop_s *P, float *const *S, const float *uf, float *grad)
     return rc;
 }
 
-// TMA-fed passes need 16-byte row strides (NZ a multiple of 4), the
+// TMA-fed passes need 16-byte row strides (a pitch of a multiple of 4), the
 // driver's tensor-map encoder and (TTI) the symmetry-axis arrays
 bool tma_usable(const prop_s *P)
 {
-    return P->g.NZ % 4 == 0 && encode_fn() != nullptr && getenv("WAVEPROP_NO_TMA") == nullptr &&
+    return P->g.PZ % 4 == 0 && !P->pipelined && encode_fn() != nullptr && getenv("WAVEPROP_NO_TMA") == nullptr &&
            (P->d.kind != PROP_TTI || (P->nrm[0] && P->nrm[1]));
 }
 

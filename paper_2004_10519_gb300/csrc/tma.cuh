@@ -105,7 +105,7 @@ WP_DEV void drain(uint64_t *full, int a, int b)
     for (int j = a < 0 ? 0 : a; j <= b; j++) mbar_wait(&full[j % NS], (uint32_t)((j / NS) & 1));
 }
 
-// 8-byte accesses (z even, NZ even: always aligned)
+// 8-byte accesses (z even, row pitch even: always aligned)
 // Bounds-checking build (WP_CHECK, selected at run time by WAVEPROP_CHECK=1):
 // every shared-memory read must lie in the CTA's dynamic shared memory, every
 // global float2 access of a field below the grid size and every TMA copy
@@ -279,13 +279,14 @@ EncodeTiled encode_fn()
     return fn;
 }
 
-// 3D map of a [NX][NY][NZ] float array, box (bz, by, 1); zero fill outside
+// 3D map of a [NX][NY][NZ] float array with rows PZ floats apart, box (bz, by,
+// 1); zero fill outside the grid, the row padding included
 bool make_map(CUtensorMap *m, const float *base, const GridDev &g, int bz, int by)
 {
     EncodeTiled fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)g.NZ, (cuuint64_t)g.NY, (cuuint64_t)g.NX};
-    cuuint64_t strides[2] = {(cuuint64_t)g.NZ * 4, (cuuint64_t)g.NZ * g.NY * 4};
+    cuuint64_t strides[2] = {(cuuint64_t)g.PZ * 4, (cuuint64_t)g.PZ * g.NY * 4};
     cuuint32_t box[3] = {(cuuint32_t)bz, (cuuint32_t)by, 1};
     cuuint32_t es[3] = {1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void *)base, dims, strides, box, es,

@@ -80,8 +80,8 @@ tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__res
         return;
     }
     const bool act = y < g.NY && z < g.NZ;
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
-    const unsigned q0 = act ? (unsigned)y * g.NZ + z : 0u;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
+    const unsigned q0 = act ? (unsigned)y * g.PZ + z : 0u;
     const float2 Z2 = make_float2(0.f, 0.f);
     float2 qp[Q], qr[Q];
 #pragma unroll
@@ -330,8 +330,8 @@ tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float
         return;
     }
     const bool act = y < g.NY && z < g.NZ;
-    const unsigned pl = (unsigned)g.NY * (unsigned)g.NZ;
-    const unsigned q0 = act ? (unsigned)y * g.NZ + z : 0u;
+    const unsigned pl = (unsigned)g.NY * (unsigned)g.PZ;
+    const unsigned q0 = act ? (unsigned)y * g.PZ + z : 0u;
     const float2 Z2 = make_float2(0.f, 0.f);
     // partial sums of the x terms for planes x .. x+2M: primed with the
     // fluxes of planes xa-M .. xa+M-1 (centred) and xa-M-1 .. xa+M-2
