@@ -331,6 +331,9 @@ std::vector<float> layer_tables(const GridDev &g, int kind);
 // planes per CTA for the x-streaming stencil kernels
 int stencil_xchunk(const GridDev &g, int sms);
 
+// the handle's row pitch (g.PZ, g.N) and pass family, from its grid and options
+void row_pitch(prop_s *P);
+
 // error helpers
 int wp_fail(prop_s *P, int code, const std::string &msg);
 // every device allocation of the library goes through wp_dev_alloc

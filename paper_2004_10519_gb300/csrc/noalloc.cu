@@ -155,9 +155,11 @@ int run(prop_s *P, const prop_desc *d, const float *const *model, const float *w
     g.NX = d->nx + 2 * d->nbl; g.NY = d->ny + 2 * d->nbl; g.NZ = d->nz + 2 * d->nbl;
     g.PZ = g.NZ;
     g.N = (long long)g.NX * g.NY * g.PZ;
+    row_pitch(P);              // padded rows as prop_create's, where they fit
     g.h = d->h; g.ih = 1.f / d->h; g.cer = 0.015f;
     if (!fd_weights(P->M, P->w.c, P->w.b)) return wp_fail(P, PROP_EINVAL, "FD weights");
-    const size_t np = (size_t)d->nx * d->ny * d->nz, N = (size_t)g.N;
+    const size_t np = (size_t)d->nx * d->ny * d->nz;
+    size_t N = (size_t)g.N;
     const int nt = d->nt;
 
     // ---- scratch layout (sizing pass first) ------------------------------
@@ -185,6 +187,15 @@ int run(prop_s *P, const prop_desc *d, const float *const *model, const float *w
     };
     Carver sizing{nullptr};
     layout(sizing);
+    if (sizing.off > WP_NOALLOC_BYTES && g.PZ != g.NZ) {     // fits with packed rows only?
+        g.PZ = g.NZ;
+        g.N = (long long)g.NX * g.NY * g.PZ;
+        N = (size_t)g.N;
+        if (int rc = sp_host_tables(P, hs.data(), nsrc, nullptr, TS)) return rc;
+        if (int rc = sp_host_tables(P, hr.data(), nrec, nullptr, TR)) return rc;
+        sizing = Carver{nullptr};
+        layout(sizing);
+    }
     if (sizing.off > WP_NOALLOC_BYTES) {
         char buf[240];
         snprintf(buf, sizeof buf,

@@ -501,7 +501,7 @@ extern "C" int prop_tile_rows(const prop_t *P) { return P ? P->tile_y : 0; }
 // into one of its own size.
 // Before and after, so 12, 281 x 267 x 193: TTI step 583 -> 350 us; so 8, 201 x
 // 171 x 139: elastic adjoint step 310 -> 136 us.
-static void row_pitch(prop_s *P)
+void row_pitch(prop_s *P)
 {
     GridDev &g = P->g;
     if (g.NZ % 4 == 0 || P->d.kind == PROP_ELASTIC2D) return;
