@@ -62,7 +62,8 @@ struct prop_s {
     std::string err;
     float vmax = 0.f;        // max model velocity used for the CFL rule
     // model (computational grid)
-    float *m = nullptr, *eps = nullptr, *del = nullptr, *th = nullptr, *ph = nullptr;   // TTI
+    // (TTI: the coupling matrix [[c1, c2], [c2, 1]], c1 = 1 + 2 eps, c2 = sqrt(1 + 2 delta))
+    float *m = nullptr, *c1 = nullptr, *c2 = nullptr, *th = nullptr, *ph = nullptr;     // TTI
     float *acw = nullptr;    // acoustic: dt^2 / m
     float *nrm[2] = {};      // TTI symmetry axis n_x, n_y (sign chosen so that n_z >= 0)
     float *bu = nullptr, *lam = nullptr, *mu = nullptr;                                 // elastic

@@ -250,7 +250,7 @@ int run(prop_s *P, const prop_desc *d, const float *const *model, const float *w
     if (int rc = layout(C)) return rc;
     int k = 0;
     if (tti) {
-        P->m = fields[k++]; P->eps = fields[k++]; P->del = fields[k++]; P->th = fields[k++]; P->ph = fields[k++];
+        P->m = fields[k++]; P->c1 = fields[k++]; P->c2 = fields[k++]; P->th = fields[k++]; P->ph = fields[k++];
         P->nrm[0] = fields[k++]; P->nrm[1] = fields[k++];
     } else {
         P->bu = fields[k++]; P->lam = fields[k++]; P->mu = fields[k++];
@@ -268,10 +268,11 @@ int run(prop_s *P, const prop_desc *d, const float *const *model, const float *w
         WP_CK(P, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         P->xchunk = stencil_xchunk(g, sms);
     }
-    float *mdst[5] = {tti ? P->m : P->bu, tti ? P->eps : P->lam, tti ? P->del : P->mu, P->th, P->ph};
+    float *mdst[5] = {tti ? P->m : P->bu, tti ? P->c1 : P->lam, tti ? P->c2 : P->mu, P->th, P->ph};
     for (int i = 0; i < nf; i++) {
         WP_CK(P, cudaMemcpyAsync(phys, hm[i].data(), np * sizeof(float), cudaMemcpyHostToDevice, P->stream));
-        k_extend(P, phys, mdst[i], (tti && i == 0) ? 1000.f : 1.f, (tti && i == 0) ? 1 : 0);
+        // TTI: m, the couplings c1 and c2, the angles (as prop_create)
+        k_extend(P, phys, mdst[i], (tti && i == 0) ? 1000.f : 1.f, tti && i < 3 ? i + 1 : 0);
     }
     if (!tti) k_lame(P);
     else k_normals(P);

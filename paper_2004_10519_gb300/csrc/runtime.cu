@@ -327,7 +327,7 @@ static void free_snaps(prop_s *P)
 
 static void free_all(prop_s *P)
 {
-    float *arrs[] = {P->m, P->eps, P->del, P->th, P->ph, P->nrm[0], P->nrm[1], P->bu, P->lam, P->mu, P->acw};
+    float *arrs[] = {P->m, P->c1, P->c2, P->th, P->ph, P->nrm[0], P->nrm[1], P->bu, P->lam, P->mu, P->acw};
     for (float *a : arrs) cudaFree(a);
     for (auto &a : P->st) cudaFree(a);
     for (auto &a : P->ast) cudaFree(a);
@@ -611,8 +611,8 @@ static int create_impl(prop_s *P, const prop_desc *d, const float *const *model)
     };
     if (d->kind == PROP_TTI) {
         WP_TRY(upload(0, P->m, 1000.f, 1));
-        WP_TRY(upload(1, P->eps, 1.f, 0));
-        WP_TRY(upload(2, P->del, 1.f, 0));
+        WP_TRY(upload(1, P->c1, 1.f, 2));
+        WP_TRY(upload(2, P->c2, 1.f, 3));
         WP_TRY(upload(3, P->th, 1.f, 0));
         WP_TRY(upload(4, P->ph, 1.f, 0));
         WP_MALLOC(P, P->nrm[0], N * sizeof(float), "symmetry axis");

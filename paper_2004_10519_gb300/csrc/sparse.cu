@@ -47,7 +47,7 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
                               float *f0, float *f1, float *f2, const float *__restrict__ gu,
                               float *grad, const int *__restrict__ tdev, const float *__restrict__ lr)
 {
-    // lam, mu: the elastic Lame parameters; for TTI (mode 3) epsilon, delta
+    // lam, mu: the elastic Lame parameters; for TTI (mode 3) the couplings c1, c2
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= ncell) return;
     if (tdev) t = *tdev;
@@ -71,7 +71,7 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
     if (mode == 3) {
         // TTI transposed step: the residual enters lam_p; keep zeta = C lam
         // (f1, f2) consistent: zeta_p += (1 + 2 eps) v, zeta_r += sqrt(1 + 2 delta) v
-        const float c1 = 1.f + 2.f * lam[q], c2 = sqrtf(1.f + 2.f * mu[q]);
+        const float c1 = lam[q], c2 = mu[q];
         f1[q] = lr ? c1 * f0[q] + c2 * lr[q] : f1[q] + c1 * v;
         f2[q] = lr ? c2 * f0[q] + lr[q] : f2[q] + c2 * v;
     } else {
@@ -120,7 +120,8 @@ __global__ void transpose_kernel(const float *__restrict__ in, float *__restrict
     }
 }
 
-// mode 0: comp = scale*phys ; 1: comp = 1/(scale*phys)^2
+// mode 0: comp = scale*phys ; 1: comp = 1/(scale*phys)^2 ; 2: 1 + 2 phys ;
+// 3: sqrt(1 + 2 phys) (the TTI couplings, once per model instead of per step)
 __global__ void extend_kernel(GridDev g, const float *__restrict__ phys, float *__restrict__ comp,
                               float scale, int mode)
 {
@@ -131,6 +132,7 @@ __global__ void extend_kernel(GridDev g, const float *__restrict__ phys, float *
               k = clampi(z - g.nbl, 0, g.pz - 1);
     const float v = phys[((long long)i * g.py + j) * g.pz + k];
     if (mode == 0) comp[q] = scale * v;
+    else if (mode >= 2) comp[q] = mode == 2 ? 1.f + 2.f * v : sqrtf(1.f + 2.f * v);
     else {
         const float s = scale * v;
         comp[q] = 1.f / (s * s);
@@ -199,13 +201,13 @@ __global__ void stack_kernel(const float *__restrict__ img, float *stack, int nx
     }
 }
 
-__global__ void zeta_kernel(long long n, const float *__restrict__ eps, const float *__restrict__ del,
+__global__ void zeta_kernel(long long n, const float *__restrict__ c1, const float *__restrict__ c2,
                             const float *__restrict__ lp, const float *__restrict__ lr,
                             float *__restrict__ zp, float *__restrict__ zr)
 {
     long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (q >= n) return;
-    const float a = 1.f + 2.f * eps[q], s = sqrtf(1.f + 2.f * del[q]);
+    const float a = c1[q], s = c2[q];
     const float p = lp[q], r = lr[q];
     zp[q] = a * p + s * r;
     zr[q] = s * p + r;
@@ -423,8 +425,8 @@ void sp_inject(prop_s *P, const SparseDev *S, const float *traces, int nt, int t
     if (S->ncell <= 0) return;
     inject_kernel<<<nblk(S->ncell), NB, 0, P->stream>>>(P->g, S->ncell, S->cell, S->cell_ptr,
                                                         S->ent_trace, S->ent_w, traces, nt, t, scale,
-                                                        mode, P->m, mode == 3 ? P->eps : P->lam,
-                                                        mode == 3 ? P->del : P->mu, f0, f1, f2,
+                                                        mode, P->m, mode == 3 ? P->c1 : P->lam,
+                                                        mode == 3 ? P->c2 : P->mu, f0, f1, f2,
                                                         grad_u, grad, tdev, lr);
     P->kern_launches++;
 }
@@ -487,7 +489,7 @@ void k_stack(prop_s *P, const float *img, float *stack, const int *gdims, const 
 
 void k_tti_zeta(prop_s *P, const float *lp, const float *lr, float *zp, float *zr)
 {
-    zeta_kernel<<<nblk(P->g.N), NB, 0, P->stream>>>(P->g.N, P->eps, P->del, lp, lr, zp, zr);
+    zeta_kernel<<<nblk(P->g.N), NB, 0, P->stream>>>(P->g.N, P->c1, P->c2, lp, lr, zp, zr);
     P->kern_launches += 1;
 }
 

@@ -174,6 +174,18 @@ WP_DEV float2 f2s(float a) { return make_float2(a, a); }
 // a - b as fma(-1, b, a): the same rounding as the subtraction
 WP_DEV float2 f2sub(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
 
+// x / a, correctly rounded, from y = RN(1/a) shared by several quotients of the
+// same divisor: q = RN(x y), corrected by its exact remainder (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor",
+// IBM J. Res. Dev. 34, 1990).  Holds while the remainder, 2^-24 of x, is a normal
+// number or zero; an infinite x gives NaN.
+WP_DEV float2 div_by(float2 x, float2 a, float2 y)
+{
+    const float2 q = f2mul(x, y);
+    const float2 r = f2fma(make_float2(-a.x, -a.y), q, x);
+    return f2fma(r, y, q);
+}
+
 constexpr int al32(int n) { return (n + 31) & ~31; }   // 128-byte aligned float offsets
 constexpr int IS = FZ * FY;                             // interior box (tile of one plane)
 

@@ -20,7 +20,7 @@ using namespace tile;
 
 template <bool ADJ>
 WP_DEV void src_pair(const GridDev &g, const float *__restrict__ p, const float *__restrict__ r,
-                     const float *__restrict__ eps, const float *__restrict__ del, int x, int y,
+                     const float *__restrict__ c1a, const float *__restrict__ c2a, int x, int y,
                      int z, float &vp, float &vr)
 {
     if (!inside(g, x, y, z)) {
@@ -33,7 +33,7 @@ WP_DEV void src_pair(const GridDev &g, const float *__restrict__ p, const float 
         vp = a;
         vr = b;
     } else {
-        const float c1 = 1.f + 2.f * __ldg(eps + q), c2 = sqrtf(1.f + 2.f * __ldg(del + q));
+        const float c1 = __ldg(c1a + q), c2 = __ldg(c2a + q);
         vp = c1 * a + c2 * b;
         vr = c2 * a + b;
     }
@@ -42,7 +42,7 @@ WP_DEV void src_pair(const GridDev &g, const float *__restrict__ p, const float 
 template <int M, int ADJ, bool RAW = false>
 __global__ void __launch_bounds__(NT, 2)
 tti_rot_p(GridDev g, FDW w, const float *__restrict__ p, const float *__restrict__ r,
-          const float *__restrict__ eps, const float *__restrict__ del, const float *__restrict__ nxa,
+          const float *__restrict__ c1a, const float *__restrict__ c2a, const float *__restrict__ nxa,
           const float *__restrict__ nya, float *__restrict__ ex, float *__restrict__ ey,
           float *__restrict__ ez, float *__restrict__ fx, float *__restrict__ fy,
           float *__restrict__ fz, int xc)
@@ -58,15 +58,15 @@ tti_rot_p(GridDev g, FDW w, const float *__restrict__ p, const float *__restrict
     hs.init([](int) { return 2; }, [](int) { return 0; }, tid);
     float qp[Q], qr[Q];
 #pragma unroll
-    for (int j = 0; j < Q - 1; j++) src_pair<ADJ>(g, p, r, eps, del, xa - M + j, y, z, qp[j], qr[j]);
+    for (int j = 0; j < Q - 1; j++) src_pair<ADJ>(g, p, r, c1a, c2a, xa - M + j, y, z, qp[j], qr[j]);
     float np_, nr_, hp[S], hr[S];
     auto fetch = [&](int x) {
-        src_pair<ADJ>(g, p, r, eps, del, x + M, y, z, np_, nr_);
+        src_pair<ADJ>(g, p, r, c1a, c2a, x + M, y, z, np_, nr_);
 #pragma unroll
         for (int k = 0; k < S; k++) {
             hp[k] = hr[k] = 0.f;
             if (hs.fld(k) >= 0)
-                src_pair<ADJ>(g, p, r, eps, del, x, y0 + hs.dy(k), z0 + hs.dz(k), hp[k], hr[k]);
+                src_pair<ADJ>(g, p, r, c1a, c2a, x, y0 + hs.dy(k), z0 + hs.dz(k), hp[k], hr[k]);
         }
     };
     fetch(xa);
@@ -139,8 +139,8 @@ template <int M, int ADJ>
 __global__ void __launch_bounds__(NT, 2)
 tti_upd_p(GridDev g, FDW w, const float *__restrict__ ex, const float *__restrict__ ey,
           const float *__restrict__ ez, const float *__restrict__ fx, const float *__restrict__ fy,
-          const float *__restrict__ fz, const float *__restrict__ m, const float *__restrict__ eps,
-          const float *__restrict__ del, const float *__restrict__ pc, const float *__restrict__ rc,
+          const float *__restrict__ fz, const float *__restrict__ m, const float *__restrict__ c1a,
+          const float *__restrict__ c2a, const float *__restrict__ pc, const float *__restrict__ rc,
           float *__restrict__ pp, float *__restrict__ rp, const float *__restrict__ up,
           const float *__restrict__ ur, float *__restrict__ grad, int *flag, int check, int xc)
 {
@@ -196,11 +196,11 @@ tti_upd_p(GridDev g, FDW w, const float *__restrict__ ex, const float *__restric
             if (hs.fld(k) >= 0) B[hs.off[k]] = hv[k];
         __syncthreads();
         const long long q = act ? gidx(g, x, y, z) : 0;
-        float mm = 1.f, e_ = 0.f, d_ = 0.f, p1 = 0.f, r1 = 0.f, p0 = 0.f, r0 = 0.f;
+        float mm = 1.f, a = 1.f, s = 1.f, p1 = 0.f, r1 = 0.f, p0 = 0.f, r0 = 0.f;
         if (act) {
             if (ADJ != 2) mm = __ldg(m + q);
-            if (ADJ != 1) d_ = __ldg(del + q);
-            if (ADJ == 0) e_ = __ldg(eps + q);
+            if (ADJ != 1) s = __ldg(c2a + q);
+            if (ADJ == 0) a = __ldg(c1a + q);
             p1 = __ldg(pc + q);
             r1 = __ldg(rc + q);
             p0 = pp[q];
@@ -226,11 +226,10 @@ tti_upd_p(GridDev g, FDW w, const float *__restrict__ ex, const float *__restric
                 // lam_p H0 p^n, g_delta (rp) += dt^2 (lam_p Hz r^n + lam_r
                 // H0 p^n) / sqrt(1 + 2 delta)
                 pp[q] = p0 + 2.f * dt2 * p1 * h0;
-                rp[q] = r0 + dt2 * (p1 * hz + r1 * h0) / sqrtf(1.f + 2.f * d_);
+                rp[q] = r0 + dt2 * (p1 * hz + r1 * h0) / s;
             } else {
             float Lp, Lr;
             if (!ADJ) {
-                const float a = 1.f + 2.f * e_, s = sqrtf(1.f + 2.f * d_);
                 Lp = a * h0 + s * hz;
                 Lr = s * h0 + hz;
             } else {
@@ -268,10 +267,10 @@ int launch(prop_s *P, float *const *S, const float *up, const float *ur, float *
                               cudaFuncSetAttribute(tti_upd_p<M, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2), true);
     (void)attr;
     prof_begin(P, ADJ ? 1 : 0);
-    tti_rot_p<M, ADJ><<<grd, blk, s1, P->stream>>>(g, P->w, S[0], S[1], P->eps, P->del, P->nrm[0], P->nrm[1],
+    tti_rot_p<M, ADJ><<<grd, blk, s1, P->stream>>>(g, P->w, S[0], S[1], P->c1, P->c2, P->nrm[0], P->nrm[1],
                                                    t[0], t[1], t[2], t[3], t[4], t[5], xc);
     tti_upd_p<M, ADJ><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[1], t[2], t[3], t[4], t[5], P->m,
-                                                   P->eps, P->del, S[0], S[1], S[2], S[3], up, ur,
+                                                   P->c1, P->c2, S[0], S[1], S[2], S[3], up, ur,
                                                    grad, P->flag, P->d.check_nan, xc);
     prof_end(P, ADJ ? 1 : 0);
     P->kern_launches += 2;
@@ -299,16 +298,16 @@ int image_aniso(prop_s *P, const float *up, const float *ur, const float *lp, co
          cudaFuncSetAttribute(tti_rot_p<M, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1),
          cudaFuncSetAttribute(tti_upd_p<M, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2), true);
     (void)attr;
-    tti_rot_p<M, 0><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, P->eps, P->del, P->nrm[0], P->nrm[1], t[0], t[1],
+    tti_rot_p<M, 0><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, P->c1, P->c2, P->nrm[0], P->nrm[1], t[0], t[1],
                                                  t[2], t[3], t[4], t[5], xc);
-    tti_upd_p<M, 2><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[1], t[2], t[3], t[4], t[5], P->m, P->eps, P->del,
+    tti_upd_p<M, 2><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[1], t[2], t[3], t[4], t[5], P->m, P->c1, P->c2,
                                                  lp, lr, ge, gd, nullptr, nullptr, nullptr, P->flag, 0, xc);
     P->kern_launches += 2;
     if (gax) {
         k_tti_zeta(P, lp, lr, t[6], t[7]);
-        tti_rot_p<M, 0, true><<<grd, blk, s1, P->stream>>>(g, P->w, t[6], t[7], P->eps, P->del, P->nrm[0],
+        tti_rot_p<M, 0, true><<<grd, blk, s1, P->stream>>>(g, P->w, t[6], t[7], P->c1, P->c2, P->nrm[0],
                                                            P->nrm[1], t[0], t[1], t[2], t[3], t[4], t[5], xc);
-        tti_rot_p<M, 0, true><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, P->eps, P->del, P->nrm[0], P->nrm[1],
+        tti_rot_p<M, 0, true><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, P->c1, P->c2, P->nrm[0], P->nrm[1],
                                                            t[8], t[9], t[10], t[11], t[12], t[13], xc);
         P->kern_launches += 2;
         const float *dz[6] = {t[0], t[1], t[2], t[3], t[4], t[5]}, *du[6] = {t[8], t[9], t[10], t[11], t[12], t[13]};

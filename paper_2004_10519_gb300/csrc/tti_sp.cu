@@ -144,8 +144,8 @@ tti_sp_rot(GridDev g, FDW w, const float *__restrict__ p, const float *__restric
 // cz_z, s0_z, sz_z (z halo); queues: c0_x, cz_x, s0_x, sz_x
 template <int M, int ADJ, int GRAD>
 __global__ void __launch_bounds__(NT, 1)
-tti_sp_upd(GridDev g, FDW w, F12 o, const float *__restrict__ m, const float *__restrict__ eps,
-           const float *__restrict__ del, const float *__restrict__ p1, const float *__restrict__ r1,
+tti_sp_upd(GridDev g, FDW w, F12 o, const float *__restrict__ m, const float *__restrict__ c1a,
+           const float *__restrict__ c2a, const float *__restrict__ p1, const float *__restrict__ r1,
            float *p0, float *r0, const float *__restrict__ up, const float *__restrict__ ur, float *grad,
            float *zp, float *zr, int *flag, int check, int xc)
 {
@@ -206,11 +206,11 @@ tti_sp_upd(GridDev g, FDW w, F12 o, const float *__restrict__ m, const float *__
             if (hs.fld(k) >= 0) B[hs.off[k]] = hv[k];
         __syncthreads();
         const long long q = act ? gidx(g, x, y, z) : 0;
-        float mm = 1.f, e_ = 0.f, d_ = 0.f, pc = 0.f, rc = 0.f, pq = 0.f, rq = 0.f;
+        float mm = 1.f, c1 = 1.f, c2 = 1.f, pc = 0.f, rc = 0.f, pq = 0.f, rq = 0.f;
         if (act) {
             mm = __ldg(m + q);
-            e_ = __ldg(eps + q);
-            d_ = __ldg(del + q);
+            c1 = __ldg(c1a + q);
+            c2 = __ldg(c2a + q);
             pc = __ldg(p1 + q);
             rc = __ldg(r1 + q);
             pq = p0[q];
@@ -236,7 +236,6 @@ tti_sp_upd(GridDev g, FDW w, F12 o, const float *__restrict__ m, const float *__
             }
             h0 *= g.ih;
             hz *= g.ih;
-            const float c1 = 1.f + 2.f * e_, c2 = sqrtf(1.f + 2.f * d_);
             const float Lp = ADJ ? h0 : c1 * h0 + c2 * hz, Lr = ADJ ? hz : c2 * h0 + hz;
             const float sd = hdt * (__ldg(g.tab + x) + syz);
             const float A = mm * (1.f + sd), Bc = mm * (1.f - sd);
@@ -284,15 +283,15 @@ int launch(prop_s *P, float *const *S, bool adjoint, const float *up, const floa
     tti_sp_rot<M><<<grd, blk, s1, P->stream>>>(g, P->w, rp_, rr_, P->nrm[0], P->nrm[1], o, xc);
     const int chk = P->d.check_nan;
     if (!adjoint)
-        tti_sp_upd<M, 0, 0><<<grd, blk, s2, P->stream>>>(g, P->w, o, P->m, P->eps, P->del, S[0], S[1], S[2],
+        tti_sp_upd<M, 0, 0><<<grd, blk, s2, P->stream>>>(g, P->w, o, P->m, P->c1, P->c2, S[0], S[1], S[2],
                                                          S[3], nullptr, nullptr, nullptr, nullptr, nullptr,
                                                          P->flag, chk, xc);
     else if (!grad)
-        tti_sp_upd<M, 1, 0><<<grd, blk, s2, P->stream>>>(g, P->w, o, P->m, P->eps, P->del, S[0], S[1], S[2],
+        tti_sp_upd<M, 1, 0><<<grd, blk, s2, P->stream>>>(g, P->w, o, P->m, P->c1, P->c2, S[0], S[1], S[2],
                                                          S[3], nullptr, nullptr, nullptr, t[6], t[7], P->flag,
                                                          chk, xc);
     else
-        tti_sp_upd<M, 1, 1><<<grd, blk, s2, P->stream>>>(g, P->w, o, P->m, P->eps, P->del, S[0], S[1], S[2],
+        tti_sp_upd<M, 1, 1><<<grd, blk, s2, P->stream>>>(g, P->w, o, P->m, P->c1, P->c2, S[0], S[1], S[2],
                                                          S[3], up, ur, grad, t[6], t[7], P->flag, chk, xc);
     P->kern_launches += 2;
     WP_CK(P, cudaGetLastError());

@@ -203,9 +203,9 @@ tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__res
 // ---------------------------------------------------------------------------
 // pass 2.  stage: [c0_y, cz_y, s0_y, sz_y (y boxes)] [c0_z, cz_z, s0_z, sz_z
 // (z boxes)] [heads c0_x, cz_x (x+M), s0_x, sz_x (x+M-1)] [m, p^n, r^n,
-// p^{n-1}, r^{n-1}, eps, delta (plane x)] (+ [u_p, u_r, g] imaging).
+// p^{n-1}, r^{n-1}, c1, c2 (plane x)] (+ [u_p, u_r, g] imaging).
 // ADJ = 2: no step; imaging of the coupling C with the forward field whose
-// fluxes were just formed: interiors [lam_p, lam_r, delta, g_eps, g_delta]
+// fluxes were just formed: interiors [lam_p, lam_r, c2, g_eps, g_delta]
 // ---------------------------------------------------------------------------
 template <int M, int ADJ, int GRAD>
 struct SUL {
@@ -372,26 +372,25 @@ tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float
             const unsigned q = x * pl + q0;
             if constexpr (L::IMG) {
                 // g_eps += 2 dt^2 lam_p H0 p^n, g_delta += dt^2 (lam_p Hz r^n + lam_r H0 p^n) / sqrt(1 + 2 delta)
-                const float2 lp = lds2(I + L::PC * IS), lr = lds2(I + L::RC * IS), d_ = lds2(I + L::DE * IS);
+                const float2 lp = lds2(I + L::PC * IS), lr = lds2(I + L::RC * IS), c2 = lds2(I + L::DE * IS);
                 const float2 ge = lds2(I + L::UP * IS), gd = lds2(I + L::UR * IS);
                 const float h0a = h0v.x * g.ih, h0b = h0v.y * g.ih, hza = hzv.x * g.ih, hzb = hzv.y * g.ih;
                 st2(grad, q, ge.x + 2.f * dt2 * lp.x * h0a, ge.y + 2.f * dt2 * lp.y * h0b);
-                st2(zp, q, gd.x + dt2 * (lp.x * hza + lr.x * h0a) / sqrtf(1.f + 2.f * d_.x),
-                    gd.y + dt2 * (lp.y * hzb + lr.y * h0b) / sqrtf(1.f + 2.f * d_.y));
+                st2(zp, q, gd.x + dt2 * (lp.x * hza + lr.x * h0a) / c2.x,
+                    gd.y + dt2 * (lp.y * hzb + lr.y * h0b) / c2.y);
             } else {
                 const float2 mm = lds2(I + L::MM * IS), p1 = lds2(I + L::PC * IS), r1 = lds2(I + L::RC * IS);
                 const float2 p0 = lds2(I + L::PP * IS), r0 = lds2(I + L::RP * IS);
-                const float2 e_ = lds2(I + L::EP * IS), d_ = lds2(I + L::DE * IS);
+                const float2 c1v = lds2(I + L::EP * IS), c2v = lds2(I + L::DE * IS);
                 const float sxv = __ldg(sx + x);
                 const float h0[2] = {h0v.x * g.ih, h0v.y * g.ih}, hz[2] = {hzv.x * g.ih, hzv.y * g.ih};
-                const float M2[2] = {mm.x, mm.y}, E2[2] = {e_.x, e_.y}, D2[2] = {d_.x, d_.y};
+                const float M2[2] = {mm.x, mm.y};
+                const float c1[2] = {c1v.x, c1v.y}, cc[2] = {c2v.x, c2v.y};
                 const float P1[2] = {p1.x, p1.y}, R1[2] = {r1.x, r1.y}, P0[2] = {p0.x, p0.y}, R0[2] = {r0.x, r0.y};
                 const float SYZ[2] = {syz0, syz1};
-                float pn[2], rn[2], Lp[2], Lr[2], c1[2], cc[2];
+                float pn[2], rn[2], Lp[2], Lr[2];
 #pragma unroll
                 for (int i = 0; i < 2; i++) {
-                    c1[i] = 1.f + 2.f * E2[i];
-                    cc[i] = sqrtf(1.f + 2.f * D2[i]);
                     Lp[i] = ADJ ? h0[i] : c1[i] * h0[i] + cc[i] * hz[i];
                     Lr[i] = ADJ ? hz[i] : cc[i] * h0[i] + hz[i];
                     const float sd = hdt * (sxv + SYZ[i]);
@@ -448,7 +447,7 @@ int sp_launch(prop_s *P, float *const *S, const float *up, const float *ur, floa
              map_of(P, o.f[fx[f]], FZ, FY, &um.h[f]);
     ok = ok && map_of(P, P->m, FZ, FY, &um.m) && map_of(P, S[0], FZ, FY, &um.pc) &&
          map_of(P, S[1], FZ, FY, &um.rc) && map_of(P, S[2], FZ, FY, &um.pp) && map_of(P, S[3], FZ, FY, &um.rp) &&
-         map_of(P, P->eps, FZ, FY, &um.e) && map_of(P, P->del, FZ, FY, &um.d);
+         map_of(P, P->c1, FZ, FY, &um.e) && map_of(P, P->c2, FZ, FY, &um.d);
     if (GRAD)
         ok = ok && map_of(P, up, FZ, FY, &um.up) && map_of(P, ur, FZ, FY, &um.ur) && map_of(P, grad, FZ, FY, &um.g);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
@@ -551,7 +550,7 @@ int sp_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp,
     for (int f = 0; f < 4; f++)
         ok = ok && map_of(P, o.f[fy[f]], B::YC, B::YR, &um.y[f]) && map_of(P, o.f[fz[f]], B::ZC, B::ZR, &um.z[f]) &&
              map_of(P, o.f[fx[f]], FZ, FY, &um.h[f]);
-    ok = ok && map_of(P, lp, FZ, FY, &um.pc) && map_of(P, lr, FZ, FY, &um.rc) && map_of(P, P->del, FZ, FY, &um.d) &&
+    ok = ok && map_of(P, lp, FZ, FY, &um.pc) && map_of(P, lr, FZ, FY, &um.rc) && map_of(P, P->c2, FZ, FY, &um.d) &&
          map_of(P, ge, FZ, FY, &um.up) && map_of(P, gd, FZ, FY, &um.ur);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
     const size_t s1 = NSTAGE * SRL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * SUL<M, 2, 0>::SZ * sizeof(float) + 64;

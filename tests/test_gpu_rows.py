@@ -125,3 +125,22 @@ def test_staggered_pair_gradient_is_still_refused():
     with pytest.raises(wp.PropError) as e:
         prop.gradient_aniso(p.wavelet, p.src, p.rec, np.zeros((p.rec.shape[0], p.nt), np.float32))
     assert e.value.code == wp.PROP_EINVAL
+
+
+@pytest.mark.parametrize("kind", ["tti", "elastic"])
+def test_noalloc_modelling_is_bitwise_the_handle(kind):
+    import ctypes as C
+    import paper_2004_10519_gb300 as wp
+    p = problem(kind, 41)
+    ref = wp.Propagator.from_problem(p).forward(p.wavelet, p.src, p.rec)
+    q = wp.PropDesc(p.kind, p.nx, p.ny, p.nz, p.nbl, p.h, p.so, p.nt, p.dt, 0.0, 0, 0, 0, 0)
+    model = p.model_list()
+    ptr = lambda a: C.c_void_p(a.ctypes.data)
+    out = np.zeros_like(ref)
+    L = wp.lib()
+    L.prop_forward_noalloc.argtypes = [C.POINTER(wp.PropDesc), C.POINTER(C.c_void_p), C.c_void_p, C.c_void_p, C.c_int,
+                                       C.c_void_p, C.c_int, C.c_void_p, C.c_void_p]
+    rc = L.prop_forward_noalloc(C.byref(q), (C.c_void_p * len(model))(*[ptr(a) for a in model]), ptr(p.wavelet),
+                                ptr(p.src), 1, ptr(p.rec), p.rec.shape[0], ptr(out), None)
+    assert rc == 0, L.prop_last_error(None)
+    np.testing.assert_array_equal(out, ref)
