@@ -37,7 +37,10 @@
  *   - Buffers may be host or device pointers (detected per pointer with
  *     cudaPointerGetAttributes).  The caller owns every buffer passed in or
  *     out; the library owns the handle and all device memory it allocates,
- *     and frees it in prop_destroy.
+ *     and frees it in prop_destroy.  Freed memory, that of a call's buffers
+ *     included, goes to a pool that the library's next allocations take it
+ *     from: at most 1/16 of the device's memory, given back to the device
+ *     when the last handle of the process is destroyed and by prop_trim.
  *   - All work is enqueued on the stream given at prop_create (NULL = the
  *     legacy default stream); every call returns after that work completed.
  *   - Negative return = error.  After PROP_EINVAL the handle stays usable;
@@ -272,7 +275,8 @@ int prop_stack_image(prop_t *p, const float *image, float *stack, const int *sta
 /* Release the handle's work arrays (wavefield state, adjoint state,
  * scratch fields, saved forward run) and keep the model: the next call
  * allocates what it needs again (the state restarts at zero).  A batch of
- * many shots can thus hold all its handles at the size of their models;
+ * many shots can thus hold all its handles at the size of their models, and
+ * the memory is free to the device's other users, the library's pool included;
  * prop_gradient_batch trims each shot after its gradient.  Synchronises the
  * handle's stream. */
 int prop_trim(prop_t *p);

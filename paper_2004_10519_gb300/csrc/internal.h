@@ -58,6 +58,7 @@ struct prop_s {
     FDW w{};
     int M = 0;
     cudaStream_t stream = nullptr;
+    int dev = 0;             // device of the handle
     bool broken = false;
     std::string err;
     float vmax = 0.f;        // max model velocity used for the CFL rule
@@ -343,6 +344,10 @@ int wp_fail(prop_s *P, int code, const std::string &msg);
 // records the failure on the handle (P may be NULL)
 int wp_dev_alloc(void **p, size_t bytes, const char *what, std::string *msg);
 int wp_malloc(prop_s *P, void **p, size_t bytes, const char *what);
+// frees what wp_dev_alloc gave (NULL-safe; synchronises the device); bytes that
+// the pool of device memory holds unused
+void wp_dev_free(void *p);
+size_t wp_dev_idle();
 // status of the device error word read back after a call: bit 3 (the
 // bounds-checking build skipped an access) -> PROP_ECUDA; bit 1 (a bounded
 // device wait expired) -> PROP_ETIMEOUT; bit 0 (NaN/Inf seen) ->

@@ -389,7 +389,7 @@ int sp_build(prop_s *P, const float *xyz, int n, const int *trace_of_point, Spar
 
 void sp_free(SparseDev *S)
 {
-    if (S->blk) cudaFree(S->blk);
+    if (S->blk) wp_dev_free(S->blk);
     *S = SparseDev{};
 }
 

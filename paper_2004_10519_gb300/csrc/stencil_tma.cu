@@ -1711,11 +1711,11 @@ TtiBatch *tti_batch_new() { return new TtiBatch(); }
 void tti_batch_free(TtiBatch *b)
 {
     if (!b) return;
-    cudaFree(b->dtiles);
-    cudaFree(b->dshots);
-    for (auto d : b->dfixed) cudaFree(d);
-    for (auto d : b->elfixed) cudaFree(d);
-    cudaFree(b->del);
+    wp_dev_free(b->dtiles);
+    wp_dev_free(b->dshots);
+    for (auto d : b->dfixed) wp_dev_free(d);
+    for (auto d : b->elfixed) wp_dev_free(d);
+    wp_dev_free(b->del);
     for (int i = 0; i < TtiBatch::NSLOT; i++) {
         if (b->elcopied[i]) {
             cudaEventSynchronize(b->elcopied[i]);
@@ -1849,7 +1849,7 @@ static int batch_tiles(TtiBatch *b, const std::vector<prop_s *> &Ps, cudaStream_
                 for (int z = 0; z < tz; z++) b->htiles.push_back(make_int4(i, z, y, c));
     }
     if (b->htiles.size() > b->tiles_cap) {
-        cudaFree(b->dtiles);
+        wp_dev_free(b->dtiles);
         b->dtiles = nullptr;
         b->tiles_cap = 0;
         if (int rc = wp_dev_alloc((void **)&b->dtiles, b->htiles.size() * sizeof(int4), "batched TTI tile table",
@@ -1884,7 +1884,7 @@ int tti_batch_fix(TtiBatch *b, const TtiBatchReq *req, int n, int slot, cudaStre
     if (int rc = tti_batch_tiles(b, req, n, st, err)) return rc;
     if ((size_t)n > b->fixed_cap) {              // every slot holds n entries
         for (auto &d : b->dfixed) {
-            cudaFree(d);
+            wp_dev_free(d);
             d = nullptr;
         }
         b->fixed_cap = n;
@@ -1976,7 +1976,7 @@ int tti_batch_step(TtiBatch *b, const TtiBatchReq *req, int n, cudaStream_t st, 
     };
     if (int rc = tti_batch_tiles(b, req, n, st, err)) return rc;
     if ((size_t)n > b->shots_cap) {
-        cudaFree(b->dshots);
+        wp_dev_free(b->dshots);
         b->dshots = nullptr;
         b->shots_cap = 0;
         if (int rc = wp_dev_alloc((void **)&b->dshots, n * sizeof(TtiShot), "batched TTI shot table", err)) return rc;
@@ -2081,7 +2081,7 @@ static int el_batch_launch(TtiBatch *b, const ElBatchReq *req, int n, cudaStream
     const int mode = req[0].mode, per = mode == 0 ? 1 : 3;
     const size_t bytes = (size_t)n * per * sizeof(ElShot);
     if (bytes > b->del_cap) {
-        cudaFree(b->del);
+        wp_dev_free(b->del);
         b->del = nullptr;
         b->del_cap = 0;
         if (int rc = wp_dev_alloc((void **)&b->del, bytes, "batched elastic shot table", err)) return rc;
@@ -2178,7 +2178,7 @@ int el_batch_fix(TtiBatch *b, const ElBatchReq *req, int n, int slot, cudaStream
     if (int rc = batch_tiles(b, Ps, st, err)) return rc;
     if ((size_t)n > b->elfixed_cap) {             // every slot holds 3n entries
         for (auto &d : b->elfixed) {
-            cudaFree(d);
+            wp_dev_free(d);
             d = nullptr;
         }
         b->elfixed_cap = n;
