@@ -70,6 +70,9 @@ struct prop_s {
     float *bu = nullptr, *lam = nullptr, *mu = nullptr;                                 // elastic
     // state: TTI 4 fields (p_cur, r_cur, p_prev, r_prev); elastic 9 fields
     float *st[9] = {};
+    // where the next forward step of the TMA-fed passes writes what is stored of
+    // its new level (TTI p, r; acoustic u; elastic v); NULL: over the oldest level
+    float *out[3] = {};
     // scratch: TTI 6 intermediates (ex ey ez fx fy fz) + 2 (zeta p, r);
     // elastic adjoint: 6 (stress-like) + 3 (weighted velocity) + 6 gradient
     // products (edges xy xz yz, faces x y z)

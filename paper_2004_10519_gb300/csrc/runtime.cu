@@ -1202,11 +1202,44 @@ static void record_rec(prop_s *P, const SparseDev &R, float *const *s, float *co
     else sp_record(P, &R, s[3], s[4], s[5], 1.f, col);
 }
 
+// true if a forward step can write the fields that are stored of a level into
+// the storage itself, which then serves as the state of the next steps, instead
+// of being copied there (16 B/point of the 116 B of a TTI step, 24 of 144 elastic,
+// 8 of 24 acoustic; 75 of 263 us a step for acoustic so 12, 60.8 M points): the
+// TMA-fed passes read and write a level through separate pointers
+static bool stores_level(const prop_s *P)
+{
+    return tma_usable(P) && !P->rdv && P->d.kind != PROP_ELASTIC2D;
+}
+
 // One forward step n of state s (record already done).  TTI/acoustic
 // pointer rotation is applied so that s[0] (TTI: s[0..1]) hold the new level
-// afterwards.
-static int fwd_step(prop_s *P, float **s, const SparseDev &S, const float *wav, int n)
+// afterwards.  store: where the stored fields of the new level go (snap_fields
+// arrays; NULL: not stored); s then points there (stores_level) or they are
+// copied.  A state that points into the storage returns to the handle's own
+// arrays with the next step that stores nothing.
+static int fwd_step(prop_s *P, float **s, const SparseDev &S, const float *wav, int n, float *store = nullptr)
 {
+    const size_t N = (size_t)P->g.N;
+    const int nf = P->d.kind == PROP_ELASTIC2D ? 0 : (int)snap_fields(P);   // fields stored of a level
+    const bool levels = P->d.kind != PROP_ELASTIC;                  // two levels, or updated in place
+    float *const *own = P->st;
+    auto is_own = [&](const float *q) {
+        for (int i = 0; i < 9; i++)
+            if (q && own[i] == q) return true;
+        return false;
+    };
+    if (stores_level(P)) {
+        float *const *old = levels ? s + nf : s;                    // what a step without P->out overwrites
+        for (int f = 0; f < nf; f++) {
+            if (store) P->out[f] = store + f * N;
+            else if (!is_own(old[f])) P->out[f] = levels && own[f] == s[f] ? own[nf + f] : own[f];
+        }
+    }
+    struct Clear {
+        prop_s *P;
+        ~Clear() { for (auto &o : P->out) o = nullptr; }
+    } clear{P};
     if (P->d.kind == PROP_TTI) {
         WP_TRY(tti_launch_step(P, s, false, nullptr, nullptr, nullptr));
         std::swap(s[0], s[2]);
@@ -1219,27 +1252,22 @@ static int fwd_step(prop_s *P, float **s, const SparseDev &S, const float *wav, 
     } else {
         WP_TRY(el_launch_step(P, s, false));
     }
+    const bool moved = P->out[0] != nullptr;
+    for (int f = 0; f < 3; f++)
+        if (P->out[f]) s[f] = P->out[f];
     inject_src(P, S, wav, n, s);
+    if (store && !moved)
+        for (int f = 0; f < nf; f++)
+            WP_CK(P, cudaMemcpyAsync(store + f * N, s[f], N * 4, cudaMemcpyDeviceToDevice, P->stream));
     prof_maybe_collect(P);
     return PROP_OK;
 }
 
-// store level `lvl` (state s holds level lvl) in full storage
-static int store_full(prop_s *P, float *const *s, int lvl)
+// full storage of level lvl: TTI and acoustic keep 1 .. nt-1, elastic 0 .. nt-1
+static float *full_slot(prop_s *P, int lvl)
 {
-    const size_t N = (size_t)P->g.N;
-    if (P->d.kind != PROP_ELASTIC) {
-        if (lvl < 1 || lvl > P->d.nt - 1) return PROP_OK;
-        float *d = snap_slot(P, lvl - 1);
-        for (size_t f = 0; f < snap_fields(P); f++)
-            WP_CK(P, cudaMemcpyAsync(d + f * N, s[f], N * 4, cudaMemcpyDeviceToDevice, P->stream));
-    } else {
-        if (lvl < 0 || lvl > P->d.nt - 1) return PROP_OK;
-        float *d = snap_slot(P, lvl);
-        for (size_t f = 0; f < snap_fields(P); f++)
-            WP_CK(P, cudaMemcpyAsync(d + f * N, s[f], N * 4, cudaMemcpyDeviceToDevice, P->stream));
-    }
-    return PROP_OK;
+    if (lvl > P->d.nt - 1) return nullptr;
+    return snap_slot(P, P->d.kind == PROP_ELASTIC ? lvl : lvl - 1);
 }
 
 // forward time loop; stage [nt][nrec]; save: keep wavefields per snap_mode
@@ -1251,18 +1279,26 @@ static int run_forward(prop_s *P, const Geometry &G, const float *wav, float *st
     WP_TRY(zero_fields(P, s, nfields(P)));
     const bool full = save && P->d.snap_mode == SNAP_FULL_FP32;
     const bool ckpt = save && !full;
-    if (full && P->d.kind == PROP_ELASTIC) WP_TRY(store_full(P, s, 0));
+    if (full && P->d.kind == PROP_ELASTIC)                // level 0 is zero
+        WP_CK(P, cudaMemsetAsync(full_slot(P, 0), 0, snap_fields(P) * (size_t)P->g.N * 4, P->stream));
     const int span = ckpt_span(P), L0 = nt - P->tail_T;   // tail: levels L0 .. nt-1
-    const size_t tl = snap_fields(P) * (size_t)P->g.N;
+    const size_t N = (size_t)P->g.N, tl = snap_fields(P) * N;
     for (int n = 0; n < nt; n++) {
         record_rec(P, G.R, s, stage + (size_t)n * G.R.n);
         if (ckpt && n % K == 0 && n < span) WP_TRY(save_checkpoint(P, n / K, s));
-        WP_TRY(fwd_step(P, s, G.S, wav, n));
-        if (full) WP_TRY(store_full(P, s, n + 1));
-        if (ckpt && P->tail_T > 0 && n + 1 >= L0 && n + 1 <= nt - 1) {
-            float *d = P->tail + (size_t)(n + 1 - L0) * tl;
-            for (size_t f = 0; f < snap_fields(P); f++)
-                WP_CK(P, cudaMemcpyAsync(d + f * P->g.N, s[f], P->g.N * 4, cudaMemcpyDeviceToDevice, P->stream));
+        float *store = full ? full_slot(P, n + 1) : nullptr;
+        if (ckpt && P->tail_T > 0 && n + 1 >= L0 && n + 1 <= nt - 1) store = P->tail + (size_t)(n + 1 - L0) * tl;
+        WP_TRY(fwd_step(P, s, G.S, wav, n, store));
+    }
+    // level nt is not stored, so it is in the handle's own arrays; level nt-1
+    // returns there from the storage
+    if (save && stores_level(P) && P->d.kind != PROP_ELASTIC) {
+        const int nf = (int)snap_fields(P);
+        for (int f = 0; f < nf; f++) {
+            float *own = P->st[f] == s[f] ? P->st[nf + f] : P->st[f];
+            if (s[nf + f] == own) continue;
+            WP_CK(P, cudaMemcpyAsync(own, s[nf + f], N * 4, cudaMemcpyDeviceToDevice, P->stream));
+            s[nf + f] = own;
         }
     }
     // the final state, in st[] order, for prop_get_state (buffers permuted)
@@ -1420,12 +1456,7 @@ static int tti_sweep(prop_s *P, const Geometry &G, const float *res, const float
             WP_CK(P, cudaMemcpyAsync(seg_slot(P, K), s[0], N * 4, cudaMemcpyDeviceToDevice, P->stream));
             WP_CK(P, cudaMemcpyAsync(seg_slot(P, K) + N, s[1], N * 4, cudaMemcpyDeviceToDevice, P->stream));
         }
-        for (int n = n0; n < E; n++) {
-            WP_TRY(fwd_step(P, s, G.S, wav, n));
-            float *d = seg_slot(P, n - n0);     // level n+1
-            WP_CK(P, cudaMemcpyAsync(d, s[0], N * 4, cudaMemcpyDeviceToDevice, P->stream));
-            WP_CK(P, cudaMemcpyAsync(d + N, s[1], N * 4, cudaMemcpyDeviceToDevice, P->stream));
-        }
+        for (int n = n0; n < E; n++) WP_TRY(fwd_step(P, s, G.S, wav, n, seg_slot(P, n - n0)));     // level n+1
         for (int k = E; k >= n0 + 1; k--) {
             const float *u = seg_slot(P, k - n0 - 1);
             WP_TRY(adj_iter(k, u, u + N));
@@ -1469,10 +1500,7 @@ static int ac_sweep(prop_s *P, const Geometry &G, const float *res, const float 
         // restore level n0 and recompute levels n0+1..E (slot i: level n0+1+i)
         float *s[2] = {P->st[0], P->st[1]};
         WP_TRY(load_checkpoint(P, j, s));
-        for (int n = n0; n < E; n++) {
-            WP_TRY(fwd_step(P, s, G.S, wav, n));
-            WP_CK(P, cudaMemcpyAsync(seg_slot(P, n - n0), s[0], N * 4, cudaMemcpyDeviceToDevice, P->stream));
-        }
+        for (int n = n0; n < E; n++) WP_TRY(fwd_step(P, s, G.S, wav, n, seg_slot(P, n - n0)));
         for (int k = E; k >= n0 + 1; k--) WP_TRY(adj_iter(k, seg_slot(P, k - n0 - 1)));
     }
     return PROP_OK;
@@ -1530,9 +1558,8 @@ static int el_sweep(prop_s *P, const Geometry &G, const float *res, const float 
         }
         return PROP_OK;
     }
-    // k = nt-1: transposed step of a zero state, then the last residual sample
+    // k = nt-1: the transposed step of a zero state is zero; the last residual sample
     WP_TRY(zero_fields(P, P->tmp + 9, 6));      // edge and face product sums
-    WP_TRY(el_launch_step(P, a, true));
     after(nt - 1);
     const int sf = (int)snap_fields(P);
     auto xs = [&](float *base, const float **out) {
@@ -1556,12 +1583,7 @@ static int el_sweep(prop_s *P, const Geometry &G, const float *res, const float 
         WP_TRY(load_checkpoint(P, j, s));
         for (int f = 0; f < sf; f++)
             WP_CK(P, cudaMemcpyAsync(seg_slot(P, 0) + f * N, s[f], N * 4, cudaMemcpyDeviceToDevice, P->stream));
-        for (int n = n0; n < E; n++) {
-            WP_TRY(fwd_step(P, s, G.S, wav, n));
-            for (int f = 0; f < sf; f++)
-                WP_CK(P, cudaMemcpyAsync(seg_slot(P, n + 1 - n0) + f * N, s[f], N * 4,
-                                         cudaMemcpyDeviceToDevice, P->stream));
-        }
+        for (int n = n0; n < E; n++) WP_TRY(fwd_step(P, s, G.S, wav, n, seg_slot(P, n + 1 - n0)));
         for (int k = E - 1; k >= n0; k--) {
             const float *x0[9], *x1[9];
             xs(seg_slot(P, k - n0), x0);
@@ -2872,12 +2894,11 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
         WP_TRY(k_sumsq(P, (const float *)tr[i].p, m, &ss));
         mis[i] = 0.5 * ss;
     }
-    // ---- adjoint sweep: k = nt - 1 (a transposed step of the zero state and
-    // the last residual sample), then the segments, last first ----
+    // ---- adjoint sweep: k = nt - 1 (the transposed step of the zero state
+    // is zero; the last residual sample), then the segments, last first ----
     for (int i = 0; i < n; i++) {
         prop_s *P = shots[i];
         float *const *a = P->ast;
-        WP_TRY(el_launch_step(P, P->ast, true));
         sp_inject(P, &G[i].R, (const float *)tr[i].p, nt, nt - 1, 1.f, 0, a[3], a[4], a[5], nullptr, nullptr);
     }
     for (int j = J - 1; j >= 0; j--) {

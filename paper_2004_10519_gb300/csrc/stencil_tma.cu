@@ -1148,12 +1148,12 @@ int el_launch(prop_s *P, float *const *S, float dt)
 {
     GridDev g = P->g;
     g.dt = dt;
-    F9 s;
-    for (int i = 0; i < 9; i++) s.f[i] = S[i];
+    F9 s;                                      // the new velocities and, in place, the stresses
+    for (int i = 0; i < 9; i++) s.f[i] = i < 3 && P->out[i] ? P->out[i] : S[i];
     const F5 o{};
     VMaps vm;
     TMaps tm;
-    if (!vmaps<M>(P, S, S + 3, &vm) || !tmaps<M>(P, S, S + 3, &tm))
+    if (!vmaps<M>(P, S, S + 3, &vm) || !tmaps<M>(P, s.f, S + 3, &tm))
         return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
     WP_TRY((launch_v<M, 0>(P, g, s, o, vm)));
     return launch_t<M, 0>(P, g, s, o, tm);
@@ -1202,6 +1202,7 @@ int tti_launch(prop_s *P, float *const *S, const float *up, const float *ur, flo
     // the rotation pass differentiates (p, r), or zeta = C lam (tmp[6], tmp[7])
     // in the transposed step
     const float *rp_ = ADJ ? t[6] : S[0], *rr_ = ADJ ? t[7] : S[1];
+    float *pn = !ADJ && P->out[0] ? P->out[0] : S[2], *rn = !ADJ && P->out[0] ? P->out[1] : S[3];
     RMaps rm;
     UMaps um;
     bool ok = map_of(P, rp_, B::RC, B::RR, &rm.p) && map_of(P, rr_, B::RC, B::RR, &rm.r) &&
@@ -1224,7 +1225,7 @@ int tti_launch(prop_s *P, float *const *S, const float *up, const float *ur, flo
     (void)attr;
     tti_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
                                                xc, P->flag);
-    tti_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[3], um, S[2], S[3], grad, t[6], t[7],
+    tti_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[3], um, pn, rn, grad, t[6], t[7],
                                                           P->flag, P->d.check_nan, xc, P->flag);
     P->kern_launches += 2;
     WP_CK(P, cudaGetLastError());
@@ -1371,7 +1372,7 @@ int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
     const size_t sb = AL<M, GRAD>::NS * AL<M, GRAD>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(acu_tma<M, GRAD>, sb);
     (void)attr;
-    acu_tma<M, GRAD><<<grd, blk, sb, P->stream>>>(g, P->w, S[0], S[1], grad, am, P->flag, P->d.check_nan, xc,
+    acu_tma<M, GRAD><<<grd, blk, sb, P->stream>>>(g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am, P->flag, P->d.check_nan, xc,
                                                   P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());

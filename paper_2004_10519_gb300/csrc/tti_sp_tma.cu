@@ -433,6 +433,7 @@ int sp_launch(prop_s *P, float *const *S, const float *up, const float *ur, floa
     // pass 1 differentiates (p, r), or zeta = C lam (tmp[6], tmp[7]) in the
     // transposed step
     const float *rp_ = ADJ ? t[6] : S[0], *rr_ = ADJ ? t[7] : S[1];
+    float *pn = !ADJ && P->out[0] ? P->out[0] : S[2], *rn = !ADJ && P->out[0] ? P->out[1] : S[3];
     SRMaps rm;
     SUMaps um;
     bool ok = map_of(P, rp_, B::RC, B::RR, &rm.p) && map_of(P, rr_, B::RC, B::RR, &rm.r) &&
@@ -455,7 +456,7 @@ int sp_launch(prop_s *P, float *const *S, const float *up, const float *ur, floa
     static const bool attr = set_smem(tti_sp_rot_tma<M>, s1) && set_smem(tti_sp_upd_tma<M, ADJ, GRAD>, s2);
     (void)attr;
     tti_sp_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, rp_, rr_, rm, o, xc, P->flag);
-    tti_sp_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, o, um, S[2], S[3], grad, t[6], t[7], P->flag,
+    tti_sp_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, o, um, pn, rn, grad, t[6], t[7], P->flag,
                                                               P->d.check_nan, xc, P->flag);
     P->kern_launches += 2;
     WP_CK(P, cudaGetLastError());
