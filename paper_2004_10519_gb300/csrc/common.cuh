@@ -40,4 +40,39 @@ WP_DEV float ldz(const float *__restrict__ f, const GridDev &g, int x, int y, in
     return (x >= 0 && x < g.NX && y >= 0 && y < g.NY && z >= 0 && z < g.NZ) ? __ldg(f + gidx(g, x, y, z)) : 0.f;
 }
 
+// one receiver: the weighted sum over its corners
+WP_DEV float record_point(const long long *__restrict__ idx, const float *__restrict__ w, int i,
+                          const float *__restrict__ f0, const float *__restrict__ f1, const float *__restrict__ f2)
+{
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+        const long long q = idx[8 * (long long)i + c];
+        const float wc = w[8 * (long long)i + c];
+        if (wc != 0.f) {
+            float v = f0[q];
+            if (f1) v += f1[q];
+            if (f2) v += f2[q];
+            s = __fmaf_rn(wc, v, s);
+        }
+    }
+    return s;
+}
+// source term of a cell: the weighted sum of its traces at time t
+WP_DEV float inject_sum(const int *__restrict__ ptr, const int *__restrict__ tr, const float *__restrict__ w,
+                        const float *__restrict__ traces, int nt, int t, int j)
+{
+    float acc = 0.f;
+    for (int e = ptr[j]; e < ptr[j + 1]; e++) acc = __fmaf_rn(w[e], traces[(long long)tr[e] * nt + t], acc);
+    return acc;
+}
+// a source term is rounded before it is added to a field (the same bits in every
+// kernel that injects)
+WP_DEV void inject_add(float &f, float coef, float acc) { f = __fadd_rn(f, __fmul_rn(coef, acc)); }
+// scale / A, A = m (1 + sig dt/2): the factor of a TTI or acoustic source term
+WP_DEV float inject_coef(const GridDev &g, float scale, float m, int x, int y, int z)
+{
+    return scale / (m * (1.f + 0.5f * tti_sigma(g, x, y, z) * g.dt));
+}
+
 WP_DEV int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }

@@ -14,6 +14,8 @@
 
 #define WP_MAXM 8   // space order up to 16
 
+constexpr int INJ_MAX = 16;  // source cells that a pass injects itself; more go through inject_kernel
+
 // Computational grid as seen by the kernels.  Index (x,y,z) -> (x*NY + y)*PZ + z.
 struct GridDev {
     int NX, NY, NZ;          // computational grid
@@ -50,6 +52,29 @@ struct SparseDev {
     int *cell_ptr = nullptr; // [ncell+1]
     int *ent_trace = nullptr;
     float *ent_w = nullptr;
+    int few = 0;             // ncell where it is at most INJ_MAX, with the cells' places
+    int few_x[INJ_MAX] = {};
+    unsigned few_o[INJ_MAX] = {};
+};
+
+// Receivers and sources of one forward step, done by the step's own passes (the
+// TMA-fed ones): CTAs beyond the tiles of the first pass sample the level that
+// the step starts from, and the threads of the last pass add the source terms to
+// the points that they have just written.
+struct RecDev {
+    int n;                   // receivers; 0: none
+    const long long *idx;
+    const float *w;
+    const float *f0, *f1, *f2;   // sampled: f0 (+ f1 + f2)
+    float *out;
+};
+struct InjDev {
+    int n, nt, t;            // cells (0: none), trace length, time index
+    float scale;
+    const int *ptr, *tr;     // entries of a cell: trace, weight
+    const float *w, *traces, *m;
+    int x[INJ_MAX];          // plane and in-plane offset of a cell
+    unsigned o[INJ_MAX];
 };
 
 struct prop_s {
@@ -73,6 +98,8 @@ struct prop_s {
     // where the next forward step of the TMA-fed passes writes what is stored of
     // its new level (TTI p, r; acoustic u; elastic v); NULL: over the oldest level
     float *out[3] = {};
+    RecDev rec{};            // receivers and sources of the next forward step
+    InjDev inj{};
     // scratch: TTI 6 intermediates (ex ey ez fx fy fz) + 2 (zeta p, r);
     // elastic adjoint: 6 (stress-like) + 3 (weighted velocity) + 6 gradient
     // products (edges xy xz yz, faces x y z)

@@ -1212,6 +1212,33 @@ static bool stores_level(const prop_s *P)
     return tma_usable(P) && !P->rdv && P->d.kind != PROP_ELASTIC2D;
 }
 
+// true if the passes of a forward step sample the receivers and add the sources
+// themselves (the TMA-fed passes of one shot)
+static bool step_has_io(const prop_s *P)
+{
+    return tma_usable(P) && !P->rdv && P->d.kind != PROP_ELASTIC2D && P->d.tti_operator == 0;
+}
+// receivers of the next step (the level that it starts from, into column n)
+static void step_receivers(prop_s *P, const SparseDev &R, float *const *s, float *col)
+{
+    const bool el = P->d.kind == PROP_ELASTIC;
+    P->rec = RecDev{R.n, R.rec_idx, R.rec_w, el ? s[3] : s[0], el ? s[4] : nullptr, el ? s[5] : nullptr, col};
+}
+// sources of the next step; false: too many cells, inject_src does it
+static bool step_sources(prop_s *P, const SparseDev &S, const float *wav, int n)
+{
+    if (!step_has_io(P) || !S.few) return false;
+    const float dt = P->g.dt;
+    InjDev I{S.few, P->d.nt, n, P->d.kind == PROP_ELASTIC ? dt : dt * dt, S.cell_ptr, S.ent_trace, S.ent_w, wav, P->m,
+             {}, {}};
+    for (int j = 0; j < S.few; j++) {
+        I.x[j] = S.few_x[j];
+        I.o[j] = S.few_o[j];
+    }
+    P->inj = I;
+    return true;
+}
+
 // One forward step n of state s (record already done).  TTI/acoustic
 // pointer rotation is applied so that s[0] (TTI: s[0..1]) hold the new level
 // afterwards.  store: where the stored fields of the new level go (snap_fields
@@ -1238,8 +1265,14 @@ static int fwd_step(prop_s *P, float **s, const SparseDev &S, const float *wav, 
     }
     struct Clear {
         prop_s *P;
-        ~Clear() { for (auto &o : P->out) o = nullptr; }
+        ~Clear()
+        {
+            for (auto &o : P->out) o = nullptr;
+            P->rec = RecDev{};
+            P->inj = InjDev{};
+        }
     } clear{P};
+    const bool injected = step_sources(P, S, wav, n);
     if (P->d.kind == PROP_TTI) {
         WP_TRY(tti_launch_step(P, s, false, nullptr, nullptr, nullptr));
         std::swap(s[0], s[2]);
@@ -1255,7 +1288,7 @@ static int fwd_step(prop_s *P, float **s, const SparseDev &S, const float *wav, 
     const bool moved = P->out[0] != nullptr;
     for (int f = 0; f < 3; f++)
         if (P->out[f]) s[f] = P->out[f];
-    inject_src(P, S, wav, n, s);
+    if (!injected) inject_src(P, S, wav, n, s);
     if (store && !moved)
         for (int f = 0; f < nf; f++)
             WP_CK(P, cudaMemcpyAsync(store + f * N, s[f], N * 4, cudaMemcpyDeviceToDevice, P->stream));
@@ -1284,7 +1317,9 @@ static int run_forward(prop_s *P, const Geometry &G, const float *wav, float *st
     const int span = ckpt_span(P), L0 = nt - P->tail_T;   // tail: levels L0 .. nt-1
     const size_t N = (size_t)P->g.N, tl = snap_fields(P) * N;
     for (int n = 0; n < nt; n++) {
-        record_rec(P, G.R, s, stage + (size_t)n * G.R.n);
+        float *col = stage + (size_t)n * G.R.n;
+        if (step_has_io(P)) step_receivers(P, G.R, s, col);
+        else record_rec(P, G.R, s, col);
         if (ckpt && n % K == 0 && n < span) WP_TRY(save_checkpoint(P, n / K, s));
         float *store = full ? full_slot(P, n + 1) : nullptr;
         if (ckpt && P->tail_T > 0 && n + 1 >= L0 && n + 1 <= nt - 1) store = P->tail + (size_t)(n + 1 - L0) * tl;

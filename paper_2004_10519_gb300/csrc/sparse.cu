@@ -24,19 +24,7 @@ __global__ void record_kernel(int n, const long long *__restrict__ idx, const fl
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (tdev) out += (long long)(*tdev) * n;
-    float s = 0.f;
-#pragma unroll
-    for (int c = 0; c < 8; c++) {
-        const long long q = idx[8 * i + c];
-        const float wc = w[8 * i + c];
-        if (wc != 0.f) {
-            float v = f0[q];
-            if (f1) v += f1[q];
-            if (f2) v += f2[q];
-            s += wc * v;
-        }
-    }
-    out[i] = scale * s;
+    out[i] = scale * record_point(idx, w, i, f0, f1, f2);
 }
 
 __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict__ cell,
@@ -51,14 +39,12 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= ncell) return;
     if (tdev) t = *tdev;
-    float acc = 0.f;
-    for (int e = ptr[j]; e < ptr[j + 1]; e++) acc += w[e] * traces[(long long)tr[e] * nt + t];
+    const float acc = inject_sum(ptr, tr, w, traces, nt, t, j);
     const long long q = cell[j];
     float coef = scale;
     if (mode == 1 || mode == 3) {
         const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY), x = (int)(q / ((long long)g.PZ * g.NY));
-        const float A = m[q] * (1.f + 0.5f * tti_sigma(g, x, y, z) * g.dt);
-        coef = scale / A;
+        coef = inject_coef(g, scale, m[q], x, y, z);
     } else if (mode == 2 || mode == 4) {
         // residual into u = g C tbar: g (3 lambda + 2 mu) on each diagonal
         // component (mode 4, the x-z plane: g (2 lambda + 2 mu) on xx, zz)
@@ -67,7 +53,7 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
         coef = scale * ((mode == 2 ? 3.f : 2.f) * lam[q] + 2.f * mu[q]) * gn;
     }
     const float v = coef * acc;
-    f0[q] += v;
+    inject_add(f0[q], coef, acc);
     if (mode == 3) {
         // TTI transposed step: the residual enters lam_p; keep zeta = C lam
         // (f1, f2) consistent: zeta_p += (1 + 2 eps) v, zeta_r += sqrt(1 + 2 delta) v
@@ -75,8 +61,8 @@ __global__ void inject_kernel(GridDev g, int ncell, const long long *__restrict_
         f1[q] = lr ? c1 * f0[q] + c2 * lr[q] : f1[q] + c1 * v;
         f2[q] = lr ? c2 * f0[q] + lr[q] : f2[q] + c2 * v;
     } else {
-        if (f1) f1[q] += v;
-        if (f2) f2[q] += v;
+        if (f1) inject_add(f1[q], coef, acc);
+        if (f2) inject_add(f2[q], coef, acc);
     }
     if (grad) grad[q] -= gu[q] * (scale * acc) / m[q];
 }
@@ -373,6 +359,14 @@ int sp_build(prop_s *P, const float *xyz, int n, const int *trace_of_point, Spar
     S->ent_w = (float *)q;
     S->n = n;
     S->ncell = (int)T.cells.size();
+    if (S->ncell <= INJ_MAX) {
+        const long long pl = (long long)P->g.NY * P->g.PZ;
+        S->few = S->ncell;
+        for (int j = 0; j < S->ncell; j++) {
+            S->few_x[j] = (int)(T.cells[j] / pl);
+            S->few_o[j] = (unsigned)(T.cells[j] % pl);
+        }
+    }
     auto cp = [&](void *dst, const void *src, size_t bytes) -> int {
         if (bytes) WP_CK(P, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, P->stream));
         return PROP_OK;

@@ -262,8 +262,10 @@ WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 
 
 template <int M, int ADJ>
 __global__ void __launch_bounds__(NTP, occ(M <= 4 ? 2 : 1))
-el_vpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ VMaps mp, int xc, int *err)
+el_vpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ VMaps mp, const __grid_constant__ RecDev rec, int xc,
+             int *err)
 {
+    if (ADJ == 0 && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
     el_vpass_body<M, ADJ>(g, w, s, o, mp, blockIdx.x, blockIdx.y, blockIdx.z, xc, err);
 }
 
@@ -437,8 +439,8 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
 }
 
 template <int M, int MODE>
-WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, const TMaps &mp, int bx,
-                          int by, int bz, int xc, int *err)
+WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, const TMaps &mp,
+                          const InjDev *inj, int bx, int by, int bz, int xc, int *err)
 {
     using L = TL<M, MODE>;
     constexpr int Q = 2 * M;
@@ -470,13 +472,20 @@ WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 
         t_plane<M, MODE>(g, w, s, o, sm + R.st * L::SZ, t, x, qvx, qvy, qvz);
         R.release(lane);
     }
+    if (MODE == 0 && inj && t.act)
+        own_sources(*inj, t.q0, xa, xb, [&](unsigned o_, int x, int j) {
+            const unsigned q = x * (unsigned)g.NY * (unsigned)g.PZ + o_;
+            const float acc = inject_sum(inj->ptr, inj->tr, inj->w, inj->traces, inj->nt, inj->t, j);
+            for (int c = 3; c < 6; c++) inject_add(s.f[c][q], inj->scale, acc);
+        });
 }
 
 template <int M, int MODE>
 __global__ void __launch_bounds__(NTP, occ(M <= 4 ? 2 : 1))
-el_tpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ TMaps mp, int xc, int *err)
+el_tpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ TMaps mp, const __grid_constant__ InjDev inj, int xc,
+             int *err)
 {
-    el_tpass_body<M, MODE>(g, w, s, o, mp, blockIdx.x, blockIdx.y, blockIdx.z, xc, err);
+    el_tpass_body<M, MODE>(g, w, s, o, mp, &inj, blockIdx.x, blockIdx.y, blockIdx.z, xc, err);
 }
 
 // batched elastic passes: per-shot entries (grid with the step's dt,
@@ -506,7 +515,7 @@ el_tpass_batch(const ElShot *__restrict__ shots, const int4 *__restrict__ tiles,
 {
     const int4 tl = tiles[blockIdx.x];
     const ElShot &S = shots[tl.x];
-    el_tpass_body<M, MODE>(S.g, w, S.s, S.o, S.tm, tl.y, tl.z, tl.w, S.xc, S.flag);
+    el_tpass_body<M, MODE>(S.g, w, S.s, S.o, S.tm, nullptr, tl.y, tl.z, tl.w, S.xc, S.flag);
 }
 
 // ---------------------------------------------------------------------------
@@ -681,8 +690,9 @@ __global__ void __launch_bounds__(NTP, occ(MODE == 2 && M > 6 ? 1 : 2))
 tti_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__restrict__ r,
             const __grid_constant__ RMaps mp, float *__restrict__ ex, float *__restrict__ ey,
             float *__restrict__ ez, float *__restrict__ fx, float *__restrict__ fy, float *__restrict__ fz,
-            F3 hh, int xc, int *err)
+            F3 hh, const __grid_constant__ RecDev rec, int xc, int *err)
 {
+    if (MODE == 0 && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
     tti_rot_body<M, MODE>(g, w, p, r, mp, ex, ey, ez, fx, fy, fz, hh, blockIdx.x, blockIdx.y, blockIdx.z, xc,
                           err);
 }
@@ -725,7 +735,8 @@ template <int M, int ADJ, int GRAD>
 WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict__ ex,
                          const float *__restrict__ fx, const UMaps &mp, float *__restrict__ pp,
                          float *__restrict__ rp, float *__restrict__ grad, float *__restrict__ zp,
-                         float *__restrict__ zr, int *flag, int check, int bx, int by, int bz, int xc, int *err)
+                         float *__restrict__ zr, int *flag, int check, const InjDev *inj, int bx, int by, int bz,
+                         int xc, int *err)
 {
     using L = UL<M, ADJ, GRAD>;
     using B = BX<M>;
@@ -875,6 +886,14 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
         }
         R.release(lane);
     }
+    if (!ADJ && inj && act)
+        own_sources(*inj, q0, xa, xb, [&](unsigned o, int x, int j) {
+            const unsigned q = x * pl + o;
+            const float acc = inject_sum(inj->ptr, inj->tr, inj->w, inj->traces, inj->nt, inj->t, j);
+            const float coef = inject_coef(g, inj->scale, __ldg(inj->m + q), x, y, (int)(o - (unsigned)y * g.PZ));
+            inject_add(pp[q], coef, acc);
+            inject_add(rp[q], coef, acc);
+        });
 }
 
 template <int M, int ADJ, int GRAD>
@@ -882,9 +901,9 @@ __global__ void __launch_bounds__(NTP, occ(2))
 tti_upd_tma(GridDev g, FDW w, const float *__restrict__ ex, const float *__restrict__ fx,
             const __grid_constant__ UMaps mp, float *__restrict__ pp, float *__restrict__ rp,
             float *__restrict__ grad, float *__restrict__ zp, float *__restrict__ zr, int *flag, int check,
-            int xc, int *err)
+            const __grid_constant__ InjDev inj, int xc, int *err)
 {
-    tti_upd_body<M, ADJ, GRAD>(g, w, ex, fx, mp, pp, rp, grad, zp, zr, flag, check, blockIdx.x, blockIdx.y,
+    tti_upd_body<M, ADJ, GRAD>(g, w, ex, fx, mp, pp, rp, grad, zp, zr, flag, check, &inj, blockIdx.x, blockIdx.y,
                                blockIdx.z, xc, err);
 }
 
@@ -923,7 +942,7 @@ tti_upd_batch(const TtiShot *__restrict__ shots, const int4 *__restrict__ tiles,
 {
     const int4 tl = tiles[blockIdx.x];
     const TtiShot &S = shots[tl.x];
-    tti_upd_body<M, ADJ, GRAD>(S.g, w, S.t[0], S.t[3], S.um, S.pn, S.rn, S.grad, S.t[6], S.t[7], S.flag, S.check,
+    tti_upd_body<M, ADJ, GRAD>(S.g, w, S.t[0], S.t[3], S.um, S.pn, S.rn, S.grad, S.t[6], S.t[7], S.flag, S.check, nullptr,
                                tl.y, tl.z, tl.w, S.xc, S.flag);
 }
 
@@ -965,8 +984,10 @@ struct AMaps {
 template <int M, int GRAD>
 __global__ void __launch_bounds__(NTP, M <= 6 ? 2 : 1)
 acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, float *__restrict__ grad,
-        const __grid_constant__ AMaps mp, int *flag, int check, int xc, int *err)
+        const __grid_constant__ AMaps mp, int *flag, int check, const __grid_constant__ RecDev rec,
+        const __grid_constant__ InjDev inj, int xc, int *err)
 {
+    if (!GRAD && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
     using L = AL<M, GRAD>;
     constexpr int Q = 2 * M + 1;
     extern __shared__ __align__(128) float sm[];
@@ -1081,8 +1102,18 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
             R.release(lane);
         }
     }
+    if (!GRAD && a0)
+#pragma unroll
+        for (int r = 0; r < 2; r++)
+            if (ar[r])
+                own_sources(inj, qr[r], xa, xb, [&](unsigned o, int x, int j) {
+                    const unsigned q = x * pl + o;
+                    const float acc = inject_sum(inj.ptr, inj.tr, inj.w, inj.traces, inj.nt, inj.t, j);
+                    const float coef = inject_coef(g, inj.scale, __ldg(inj.m + q), x, ya + r,
+                                                   (int)(o - (unsigned)(ya + r) * g.PZ));
+                    inject_add(u0[q], coef, acc);
+                });
 }
-
 
 // descriptors of the velocity pass: velocities v[3], stress-like fields
 // sig[6] (xx yy zz xy xz yz)
@@ -1124,8 +1155,10 @@ int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const VMaps 
     const size_t sm = NSTAGE * VL<M>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(el_vpass_tma<M, ADJ>, sm);
     (void)attr;
-    el_vpass_tma<M, ADJ><<<el_grid(P), dim3(TZ2, FY + 2, 1), sm, P->stream>>>(g, P->w, s, o, vm, P->xchunk,
-                                                                                P->flag);
+    dim3 grd = el_grid(P), blk(TZ2, FY + 2, 1);
+    const RecDev rec = ADJ ? RecDev{} : P->rec;
+    grd.z += receiver_layers(rec, grd, blk);
+    el_vpass_tma<M, ADJ><<<grd, blk, sm, P->stream>>>(g, P->w, s, o, vm, rec, P->xchunk, P->flag);
     P->kern_launches++;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1136,8 +1169,8 @@ int launch_t(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const TMaps 
     const size_t sm = NSTAGE * TL<M, MODE>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(el_tpass_tma<M, MODE>, sm);
     (void)attr;
-    el_tpass_tma<M, MODE><<<el_grid(P), dim3(TZ2, FY + 2, 1), sm, P->stream>>>(g, P->w, s, o, tm, P->xchunk,
-                                                                                 P->flag);
+    el_tpass_tma<M, MODE><<<el_grid(P), dim3(TZ2, FY + 2, 1), sm, P->stream>>>(
+        g, P->w, s, o, tm, MODE == 0 ? P->inj : InjDev{}, P->xchunk, P->flag);
     P->kern_launches++;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1223,10 +1256,13 @@ int tti_launch(prop_s *P, float *const *S, const float *up, const float *ur, flo
                  s2 = NSTAGE * UL<M, ADJ, GRAD>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(tti_rot_tma<M>, s1) && set_smem(tti_upd_tma<M, ADJ, GRAD>, s2);
     (void)attr;
-    tti_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
-                                               xc, P->flag);
+    const RecDev rec = ADJ ? RecDev{} : P->rec;
+    const dim3 grd1(grd.x, grd.y, grd.z + receiver_layers(rec, grd, blk));
+    tti_rot_tma<M><<<grd1, blk, s1, P->stream>>>(g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
+                                                rec, xc, P->flag);
     tti_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[3], um, pn, rn, grad, t[6], t[7],
-                                                          P->flag, P->d.check_nan, xc, P->flag);
+                                                          P->flag, P->d.check_nan, ADJ ? InjDev{} : P->inj, xc,
+                                                          P->flag);
     P->kern_launches += 2;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1316,9 +1352,9 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
     static const bool attr = set_smem(tti_rot_tma<M>, s1) && set_smem(tti_upd_tma<M, 2, 0>, s2);
     (void)attr;
     tti_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
-                                               xc, P->flag);
+                                               RecDev{}, xc, P->flag);
     tti_upd_tma<M, 2, 0><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[3], um, nullptr, nullptr, ge, gd, nullptr,
-                                                     P->flag, 0, xc, P->flag);
+                                                     P->flag, 0, InjDev{}, xc, P->flag);
     P->kern_launches += 2;
     if (gax) {
         RMaps rz;
@@ -1329,9 +1365,9 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
         static const bool attr_raw = set_smem(tti_rot_tma<M, 1>, s1);
         (void)attr_raw;
         tti_rot_tma<M, 1><<<grd, blk, s1, P->stream>>>(g, P->w, t[6], t[7], rz, t[0], t[1], t[2], t[3], t[4], t[5],
-                                                       F3{}, xc, P->flag);
+                                                       F3{}, RecDev{}, xc, P->flag);
         tti_rot_tma<M, 1><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, rm, t[8], t[9], t[10], t[11], t[12], t[13],
-                                                       F3{}, xc, P->flag);
+                                                       F3{}, RecDev{}, xc, P->flag);
         AxisIn ai;
         for (int c = 0; c < 6; c++) {
             ai.dz[c] = t[c];
@@ -1372,8 +1408,10 @@ int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
     const size_t sb = AL<M, GRAD>::NS * AL<M, GRAD>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(acu_tma<M, GRAD>, sb);
     (void)attr;
-    acu_tma<M, GRAD><<<grd, blk, sb, P->stream>>>(g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am, P->flag, P->d.check_nan, xc,
-                                                  P->flag);
+    const RecDev rec = GRAD ? RecDev{} : P->rec;
+    grd.z += receiver_layers(rec, grd, blk);
+    acu_tma<M, GRAD><<<grd, blk, sb, P->stream>>>(g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am, P->flag,
+                                                  P->d.check_nan, rec, GRAD ? InjDev{} : P->inj, xc, P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1419,7 +1457,7 @@ int raw_half(prop_s *P, const float *p, const float *r, float *const *dp, float 
     static const bool attr = set_smem(tti_rot_tma<M, 2>, s1);
     (void)attr;
     tti_rot_tma<M, 2><<<grd, blk, s1, P->stream>>>(g, P->w, p, r, rm, dp[0], dp[1], dp[2], dr[0], dr[1], dr[2],
-                                                   F3{{h[0], h[1], h[2]}}, xc, P->flag);
+                                                   F3{{h[0], h[1], h[2]}}, RecDev{}, xc, P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;

@@ -213,6 +213,34 @@ WP_DEV void zwin(const float *row, int cz, float (&w)[2 * M + 2])
     }
 }
 
+// The CTAs of a pass beyond its x chunks (blockIdx.z >= nz) sample the receivers
+// of the step, one per thread; true for such a CTA.  Saves a launch per step
+// that only reads what the pass reads.
+WP_DEV bool sample_receivers(const RecDev &r, int nz)
+{
+    if ((int)blockIdx.z < nz) return false;
+    const int nth = blockDim.x * blockDim.y, tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const int i = (((int)blockIdx.z - nz) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const long long k = (long long)i * nth + tid;
+    if (k < r.n) r.out[k] = record_point(r.idx, r.w, (int)k, r.f0, r.f1, r.f2);
+    return true;
+}
+// the z layers of CTAs that this takes
+inline unsigned receiver_layers(const RecDev &r, dim3 grd, dim3 blk)
+{
+    const long long ctas = ((long long)r.n + blk.x * blk.y - 1) / (blk.x * blk.y), layer = (long long)grd.x * grd.y;
+    return (unsigned)((ctas + layer - 1) / layer);
+}
+// Source terms of the step at the points of a column pair (in-plane offset q0,
+// planes [xa, xb)) that this thread has written: f(cell offset, plane, j) for
+// each of the cells among them.  A handful of compares per thread and chunk.
+template <class F>
+WP_DEV void own_sources(const InjDev &I, unsigned q0, int xa, int xb, F f)
+{
+    for (int j = 0; j < I.n; j++)
+        if (I.o[j] - q0 < 2u && I.x[j] >= xa && I.x[j] < xb) f(I.o[j], I.x[j], j);
+}
+
 // Producer/consumer plane ring.  full[s] completes when the copies of a
 // stage have landed (one arrive with the byte count + the TMA bytes);
 // empty[s] when every consumer warp has finished reading it (one arrive per
