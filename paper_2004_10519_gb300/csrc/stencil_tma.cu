@@ -238,11 +238,13 @@ WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 
     const int xa = bz * xc, xb = min(xa + xc, g.NX), nit = xb - xa;
     auto issue = [&](int x, int st) { v_issue<M>(mp, sm + st * L::SZ, &bars[st], z0, y0, x, g.NX); };
     Ring R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -452,11 +454,13 @@ WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 
     const int xa = bz * xc, xb = min(xa + xc, g.NX), nit = xb - xa;
     auto issue = [&](int x, int st) { t_issue<M, MODE>(mp, sm + st * L::SZ, &bars[st], z0, y0, x, g.NX); };
     Ring R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -575,11 +579,13 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
         tma3(S + L::ON + IS, &mp.ny, z0, y0, x, bar);
     };
     RingN<L::NS> R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -778,11 +784,13 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
         }
     };
     Ring R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -1012,11 +1020,13 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
         }
     };
     RingN<L::NS> R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -1158,7 +1168,7 @@ int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const VMaps 
     dim3 grd = el_grid(P), blk(TZ2, FY + 2, 1);
     const RecDev rec = ADJ ? RecDev{} : P->rec;
     grd.z += receiver_layers(rec, grd, blk);
-    el_vpass_tma<M, ADJ><<<grd, blk, sm, P->stream>>>(g, P->w, s, o, vm, rec, P->xchunk, P->flag);
+    launch_pass(el_vpass_tma<M, ADJ>, grd, blk, sm, P->stream, g, P->w, s, o, vm, rec, P->xchunk, P->flag);
     P->kern_launches++;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1169,8 +1179,7 @@ int launch_t(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const TMaps 
     const size_t sm = NSTAGE * TL<M, MODE>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(el_tpass_tma<M, MODE>, sm);
     (void)attr;
-    el_tpass_tma<M, MODE><<<el_grid(P), dim3(TZ2, FY + 2, 1), sm, P->stream>>>(
-        g, P->w, s, o, tm, MODE == 0 ? P->inj : InjDev{}, P->xchunk, P->flag);
+    launch_pass(el_tpass_tma<M, MODE>, el_grid(P), dim3(TZ2, FY + 2, 1), sm, P->stream, g, P->w, s, o, tm, MODE == 0 ? P->inj : InjDev{}, P->xchunk, P->flag);
     P->kern_launches++;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1258,9 +1267,9 @@ int tti_launch(prop_s *P, float *const *S, const float *up, const float *ur, flo
     (void)attr;
     const RecDev rec = ADJ ? RecDev{} : P->rec;
     const dim3 grd1(grd.x, grd.y, grd.z + receiver_layers(rec, grd, blk));
-    tti_rot_tma<M><<<grd1, blk, s1, P->stream>>>(g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
+    launch_pass(tti_rot_tma<M>, grd1, blk, s1, P->stream, g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
                                                 rec, xc, P->flag);
-    tti_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[3], um, pn, rn, grad, t[6], t[7],
+    launch_pass(tti_upd_tma<M, ADJ, GRAD>, grd, blk, s2, P->stream, g, P->w, t[0], t[3], um, pn, rn, grad, t[6], t[7],
                                                           P->flag, P->d.check_nan, ADJ ? InjDev{} : P->inj, xc,
                                                           P->flag);
     P->kern_launches += 2;
@@ -1351,9 +1360,9 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
     const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * UL<M, 2, 0>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(tti_rot_tma<M>, s1) && set_smem(tti_upd_tma<M, 2, 0>, s2);
     (void)attr;
-    tti_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
+    launch_pass(tti_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
                                                RecDev{}, xc, P->flag);
-    tti_upd_tma<M, 2, 0><<<grd, blk, s2, P->stream>>>(g, P->w, t[0], t[3], um, nullptr, nullptr, ge, gd, nullptr,
+    launch_pass(tti_upd_tma<M, 2, 0>, grd, blk, s2, P->stream, g, P->w, t[0], t[3], um, nullptr, nullptr, ge, gd, nullptr,
                                                      P->flag, 0, InjDev{}, xc, P->flag);
     P->kern_launches += 2;
     if (gax) {
@@ -1364,9 +1373,9 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
         if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
         static const bool attr_raw = set_smem(tti_rot_tma<M, 1>, s1);
         (void)attr_raw;
-        tti_rot_tma<M, 1><<<grd, blk, s1, P->stream>>>(g, P->w, t[6], t[7], rz, t[0], t[1], t[2], t[3], t[4], t[5],
+        launch_pass(tti_rot_tma<M, 1>, grd, blk, s1, P->stream, g, P->w, t[6], t[7], rz, t[0], t[1], t[2], t[3], t[4], t[5],
                                                        F3{}, RecDev{}, xc, P->flag);
-        tti_rot_tma<M, 1><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, rm, t[8], t[9], t[10], t[11], t[12], t[13],
+        launch_pass(tti_rot_tma<M, 1>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[8], t[9], t[10], t[11], t[12], t[13],
                                                        F3{}, RecDev{}, xc, P->flag);
         AxisIn ai;
         for (int c = 0; c < 6; c++) {
@@ -1410,7 +1419,7 @@ int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
     (void)attr;
     const RecDev rec = GRAD ? RecDev{} : P->rec;
     grd.z += receiver_layers(rec, grd, blk);
-    acu_tma<M, GRAD><<<grd, blk, sb, P->stream>>>(g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am, P->flag,
+    launch_pass(acu_tma<M, GRAD>, grd, blk, sb, P->stream, g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am, P->flag,
                                                   P->d.check_nan, rec, GRAD ? InjDev{} : P->inj, xc, P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());
@@ -1456,7 +1465,7 @@ int raw_half(prop_s *P, const float *p, const float *r, float *const *dp, float 
     const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(tti_rot_tma<M, 2>, s1);
     (void)attr;
-    tti_rot_tma<M, 2><<<grd, blk, s1, P->stream>>>(g, P->w, p, r, rm, dp[0], dp[1], dp[2], dr[0], dr[1], dr[2],
+    launch_pass(tti_rot_tma<M, 2>, grd, blk, s1, P->stream, g, P->w, p, r, rm, dp[0], dp[1], dp[2], dr[0], dr[1], dr[2],
                                                    F3{{h[0], h[1], h[2]}}, RecDev{}, xc, P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());

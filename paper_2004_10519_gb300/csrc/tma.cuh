@@ -213,12 +213,22 @@ WP_DEV void zwin(const float *row, int cz, float (&w)[2 * M + 2])
     }
 }
 
+// Programmatic dependent launch of the passes (launch_pass): a pass's CTAs may
+// start when every CTA of the kernel before it has, set up their barriers, and
+// wait here, before they touch anything in memory, until that kernel has
+// completed and its writes are visible.  Hides the launch latency and the
+// prologue behind the last CTAs of the pass before.  No effect in a kernel
+// that was launched without the attribute.
+WP_DEV void pass_begins() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+WP_DEV void pass_waits() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // The CTAs of a pass beyond its x chunks (blockIdx.z >= nz) sample the receivers
 // of the step, one per thread; true for such a CTA.  Saves a launch per step
 // that only reads what the pass reads.
 WP_DEV bool sample_receivers(const RecDev &r, int nz)
 {
     if ((int)blockIdx.z < nz) return false;
+    pass_waits();
     const int nth = blockDim.x * blockDim.y, tid = threadIdx.y * blockDim.x + threadIdx.x;
     const int i = (((int)blockIdx.z - nz) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     const long long k = (long long)i * nth + tid;
@@ -346,6 +356,23 @@ bool map_of(prop_s *P, const float *base, int bz, int by, CUtensorMap *out)
     }
     *out = it->second;
     return true;
+}
+
+// launch of a pass whose kernel begins with pass_begins and pass_waits
+template <class... A, class... B>
+void launch_pass(void (*kernel)(A...), dim3 grd, dim3 blk, size_t smem, cudaStream_t st, B... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grd;
+    c.blockDim = blk;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, static_cast<A>(args)...);     // errors: cudaGetLastError by the caller
 }
 
 template <class K>

@@ -70,11 +70,13 @@ tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__res
         tma3(S + L::OXN, &mp.nxi, z0, y0, min(x + 1, g.NX - 1), bar);
     };
     Ring R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -320,11 +322,13 @@ tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float
         }
     };
     Ring R(bars);
+    pass_begins();
     if (lead) {
         R.init();
         ck_begin(g.N, err);
     }
     __syncthreads();
+    pass_waits();
     if (ty >= FY) {                                       // producer warp
         if (lane == 0) R.produce(xa, nit, issue, err);
         return;
@@ -455,8 +459,8 @@ int sp_launch(prop_s *P, float *const *S, const float *up, const float *ur, floa
     const size_t s1 = NSTAGE * SRL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * SUL<M, ADJ, GRAD>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(tti_sp_rot_tma<M>, s1) && set_smem(tti_sp_upd_tma<M, ADJ, GRAD>, s2);
     (void)attr;
-    tti_sp_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, rp_, rr_, rm, o, xc, P->flag);
-    tti_sp_upd_tma<M, ADJ, GRAD><<<grd, blk, s2, P->stream>>>(g, P->w, o, um, pn, rn, grad, t[6], t[7], P->flag,
+    launch_pass(tti_sp_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, rp_, rr_, rm, o, xc, P->flag);
+    launch_pass(tti_sp_upd_tma<M, ADJ, GRAD>, grd, blk, s2, P->stream, g, P->w, o, um, pn, rn, grad, t[6], t[7], P->flag,
                                                               P->d.check_nan, xc, P->flag);
     P->kern_launches += 2;
     WP_CK(P, cudaGetLastError());
@@ -557,8 +561,8 @@ int sp_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp,
     const size_t s1 = NSTAGE * SRL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * SUL<M, 2, 0>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(tti_sp_rot_tma<M>, s1) && set_smem(tti_sp_upd_tma<M, 2, 0>, s2);
     (void)attr;
-    tti_sp_rot_tma<M><<<grd, blk, s1, P->stream>>>(g, P->w, up, ur, rm, o, xc, P->flag);
-    tti_sp_upd_tma<M, 2, 0><<<grd, blk, s2, P->stream>>>(g, P->w, o, um, nullptr, nullptr, ge, gd, nullptr, P->flag,
+    launch_pass(tti_sp_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, o, xc, P->flag);
+    launch_pass(tti_sp_upd_tma<M, 2, 0>, grd, blk, s2, P->stream, g, P->w, o, um, nullptr, nullptr, ge, gd, nullptr, P->flag,
                                                          0, xc, P->flag);
     P->kern_launches += 2;
     WP_CK(P, cudaGetLastError());
