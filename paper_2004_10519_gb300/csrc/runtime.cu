@@ -607,7 +607,7 @@ extern "C" int prop_tile_rows(const prop_t *P) { return P ? P->tile_y : 0; }
 // bytes; rows of another length get up to three floats of padding, so that they
 // run there too instead of on the pipelined passes.  Left as they are: rows so
 // short that the padding would be more than an eighth of them, grids that the
-// padding would take to 2^32 elements, 2D, and where a last bit of a wavefield
+// padding would take to 2^32 elements, and where a last bit of a wavefield
 // shows and the two families differ in it (the centred TTI passes do not): the
 // staggered-pair operators, whose FP32 error grows with the steps, and elastic
 // and acoustic handles with 16-bit checkpoints, whose rounding turns such a bit
@@ -617,9 +617,9 @@ extern "C" int prop_tile_rows(const prop_t *P) { return P ? P->tile_y : 0; }
 void row_pitch(prop_s *P)
 {
     GridDev &g = P->g;
-    if (g.NZ % 4 == 0 || P->d.kind == PROP_ELASTIC2D) return;
+    if (g.NZ % 4 == 0) return;
     const bool ckpt16 = P->d.snap_mode == SNAP_CKPT_BF16 || P->d.snap_mode == SNAP_CKPT_FP16;
-    P->pipelined = P->d.kind == PROP_TTI ? P->d.tti_operator == 1 : ckpt16;
+    P->pipelined = P->d.kind == PROP_TTI ? P->d.tti_operator == 1 : P->d.kind != PROP_ELASTIC2D && ckpt16;
     const int pz = (g.NZ + 3) / 4 * 4;
     const long long n = (long long)g.NX * g.NY * pz;
     if (P->pipelined || 8 * (pz - g.NZ) > g.NZ || n >= (1LL << 32)) return;
@@ -1216,20 +1216,22 @@ static bool stores_level(const prop_s *P)
 // themselves (the TMA-fed passes of one shot)
 static bool step_has_io(const prop_s *P)
 {
-    return tma_usable(P) && !P->rdv && P->d.kind != PROP_ELASTIC2D && P->d.tti_operator == 0;
+    return tma_usable(P) && !P->rdv && P->d.tti_operator == 0;
 }
 // receivers of the next step (the level that it starts from, into column n)
 static void step_receivers(prop_s *P, const SparseDev &R, float *const *s, float *col)
 {
-    const bool el = P->d.kind == PROP_ELASTIC;
-    P->rec = RecDev{R.n, R.rec_idx, R.rec_w, el ? s[3] : s[0], el ? s[4] : nullptr, el ? s[5] : nullptr, col};
+    RecDev r{R.n, R.rec_idx, R.rec_w, s[0], nullptr, nullptr, col};
+    if (P->d.kind == PROP_ELASTIC) r.f0 = s[3], r.f1 = s[4], r.f2 = s[5];
+    if (P->d.kind == PROP_ELASTIC2D) r.f0 = s[2], r.f1 = s[3];
+    P->rec = r;
 }
 // sources of the next step; false: too many cells, inject_src does it
 static bool step_sources(prop_s *P, const SparseDev &S, const float *wav, int n)
 {
     if (!step_has_io(P) || !S.few) return false;
     const float dt = P->g.dt;
-    InjDev I{S.few, P->d.nt, n, P->d.kind == PROP_ELASTIC ? dt : dt * dt, S.cell_ptr, S.ent_trace, S.ent_w, wav, P->m,
+    InjDev I{S.few, P->d.nt, n, P->d.kind == PROP_ELASTIC || P->d.kind == PROP_ELASTIC2D ? dt : dt * dt, S.cell_ptr, S.ent_trace, S.ent_w, wav, P->m,
              {}, {}};
     for (int j = 0; j < S.few; j++) {
         I.x[j] = S.few_x[j];
