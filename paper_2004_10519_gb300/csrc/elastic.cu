@@ -232,12 +232,14 @@ el_face2_kernel(GridDev g, Fields9 s, Fields9 xf0, Fields9 xf1, const float *__r
     const float2 u0 = ld(s.f[0], q), u1 = ld(s.f[1], q), u2 = ld(s.f[2], q);
     const float2 a0 = ld(xf0.f[0], q), a1 = ld(xf0.f[1], q), a2 = ld(xf0.f[2], q);
     const float2 c0 = ld(xf1.f[0], q), c1 = ld(xf1.f[1], q), c2 = ld(xf1.f[2], q);
-    st(f0, q, u0.x * (c0.x / (gxh * gyn * gzn0) - a0.x) / (0.5f * (b0.x + bX.x)),
-       u0.y * (c0.y / (gxh * gyn * gzn1) - a0.y) / (0.5f * (b0.y + bX.y)));
-    st(f1, q, u1.x * (c1.x / (gxn * gyh * gzn0) - a1.x) / (0.5f * (b0.x + bY.x)),
-       u1.y * (c1.y / (gxn * gyh * gzn1) - a1.y) / (0.5f * (b0.y + bY.y)));
-    st(f2, q, u2.x * (c2.x / (gxn * gyn * gzh0) - a2.x) / (0.5f * (b0.x + b0.y)),
-       u2.y * (c2.y / (gxn * gyn * gzh1) - a2.y) / (0.5f * (b0.y + bz2)));
+    // v^{k+1} - g v^k, the small difference of nearly equal values, in one fused
+    // operation; the quotient by g b_avg needs no more than its few last bits
+    auto face = [](float u, float v1, float v0, float gg, float b2) {
+        return u * __fdividef(__fmaf_rn(-gg, v0, v1), 0.5f * gg * b2);
+    };
+    st(f0, q, face(u0.x, c0.x, a0.x, gxh * gyn * gzn0, b0.x + bX.x), face(u0.y, c0.y, a0.y, gxh * gyn * gzn1, b0.y + bX.y));
+    st(f1, q, face(u1.x, c1.x, a1.x, gxn * gyh * gzn0, b0.x + bY.x), face(u1.y, c1.y, a1.y, gxn * gyh * gzn1, b0.y + bY.y));
+    st(f2, q, face(u2.x, c2.x, a2.x, gxn * gyn * gzh0, b0.x + b0.y), face(u2.y, c2.y, a2.y, gxn * gyn * gzh1, b0.y + bz2));
 }
 
 // gather of the scattered products: a node receives 1/4 of each of the 4
@@ -554,51 +556,39 @@ int launch_adj_grad(prop_s *P, float *const *S, const float *const *xk, const fl
     return PROP_OK;
 }
 
-// the same transposed step with imaging on the TMA-fed passes: pointwise
-// tapering and stiffness, three streaming passes (velocity, imaging, stress;
-// stencil_tma.cu), pointwise face products, gather
+// the same transposed step with imaging on the TMA-fed passes, from t = g tbar in
+// S[3..8] and sigma = C t in tmp[0..5]: three streaming passes (velocity, imaging,
+// stress; stencil_tma.cu), the last of which leaves t and sigma of the next step
+// (a pointwise kernel of 80 B/point did that, the pass has 32 more), and the
+// pointwise face products, whose twelve divisions a pair of points took twice the
+// time of their 64 B/point.  Forward and transposed step at 200^3, so 8: 747 ->
+// 615 us.
 int launch_adj_grad_tma(prop_s *P, float *const *S, const float *const *xk, const float *const *xk1,
                         float *const *gr)
 {
     const GridDev &g = P->g;
-    dim3 blk(TZ, TY, 1), grd((g.NZ + TZ - 1) / TZ, (g.NY + TY - 1) / TY, g.NX);
-    Fields9 s, sg, f0, f1;
+    Fields9 s, f0, f1;
     for (int i = 0; i < 9; i++) {
         s.f[i] = S[i];
-        sg.f[i] = P->tmp[i];
         f0.f[i] = const_cast<float *>(xk[i]);
         f1.f[i] = const_cast<float *>(xk1[i]);
     }
     float *const *pr = P->tmp + 9;   // edge products pr[0..2], face products pr[3..5]
     prof_begin(P, 4);
-    el_adj_pre_kernel<<<grd, blk, 0, P->stream>>>(g, s, sg, P->lam, P->mu);
     WP_TRY(el_adj_grad_tma(P, S, P->tmp, P->tmp + 6, xk1, gr, pr));
     el_face2_kernel<<<dim3((g.NZ + 63) / 64, (g.NY + 7) / 8, g.NX), dim3(32, 8, 1), 0, P->stream>>>(
         g, s, f0, f1, P->bu, pr[3], pr[4], pr[5]);
     prof_end(P, 4);
-    P->kern_launches += 2;
+    P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
 }
 
 }  // namespace
 
-// the pointwise kernels before and after the three TMA passes of a
-// transposed step with imaging, on a given stream (batched shots: the
-// passes are shared, these run per shot)
-void el_adj_pre_launch(prop_s *P, float *const *S, cudaStream_t st)
-{
-    const GridDev &g = P->g;
-    dim3 blk(TZ, TY, 1), grd((g.NZ + TZ - 1) / TZ, (g.NY + TY - 1) / TY, g.NX);
-    Fields9 s, sg;
-    for (int i = 0; i < 9; i++) {
-        s.f[i] = S[i];
-        sg.f[i] = P->tmp[i];
-    }
-    el_adj_pre_kernel<<<grd, blk, 0, st>>>(g, s, sg, P->lam, P->mu);
-    P->kern_launches += 1;
-}
-
+// the face products after the three TMA passes of a transposed step with
+// imaging, on a given stream (batched shots: the passes are shared, this runs per
+// shot)
 void el_face2_launch(prop_s *P, float *const *S, const float *const *xk, const float *const *xk1, cudaStream_t st)
 {
     const GridDev &g = P->g;

@@ -271,8 +271,7 @@ int el_batch_step(TtiBatch *b, const ElBatchReq *req, int n, cudaStream_t stream
 // may be captured
 int el_batch_fix(TtiBatch *b, const ElBatchReq *req, int n, int slot, cudaStream_t stream, std::string *err);
 int el_batch_launch_fixed(TtiBatch *b, int slot, cudaStream_t stream);
-// per-shot pointwise kernels of the batched transposed elastic step (elastic.cu)
-void el_adj_pre_launch(prop_s *P, float *const *S, cudaStream_t st);
+// per-shot pointwise kernel of the batched transposed elastic step (elastic.cu)
 void el_face2_launch(prop_s *P, float *const *S, const float *const *xk, const float *const *xk1, cudaStream_t st);
 int rdv_el_step(prop_s *P, const ElBatchReq &r);
 // a TTI step of a shot taking part in a rendezvous (runtime.cu): waits for
@@ -317,6 +316,11 @@ void sp_inject(prop_s *P, const SparseDev *S, const float *traces, int nt, int t
 // (trace of tbar from s = C tbar)
 void sp_record_trace_s(prop_s *P, const SparseDev *S, const float *f0, const float *f1,
                        const float *f2, float scale, float *out_col);
+// residual into t = g tbar (t[0..2], the diagonal) and sigma = C t (sg[0..2]); and
+// the trace of tbar sampled from t
+void sp_inject_t(prop_s *P, const SparseDev *S, const float *traces, int nt, int t, float *const *tt, float *const *sg,
+                 const int *tdev = nullptr);
+void sp_record_trace_t(prop_s *P, const SparseDev *S, float *const *tt, float scale, float *out_col);
 void sp_transpose(prop_s *P, const float *in_tn, float *out_nt, int n, int nt);
 
 // misc kernels

@@ -1577,7 +1577,10 @@ static int el_sweep(prop_s *P, const Geometry &G, const float *res, const float 
     WP_TRY(zero_fields(P, a, 9));
     if (srcstage) WP_CK(P, cudaMemsetAsync(srcstage, 0, sizeof(float) * (size_t)nt * G.S.n, P->stream));
     auto after = [&](int k) {
-        if (k >= 1) {
+        if (k >= 1 && tma_usable(P)) {               // the passes keep t = g tbar and sigma = C t (tmp[0..2])
+            sp_inject_t(P, &G.R, res, nt, k, a + 3, P->tmp);
+            if (srcstage) sp_record_trace_t(P, &G.S, a + 3, P->g.dt, srcstage + (size_t)(k - 1) * G.S.n);
+        } else if (k >= 1) {
             inject_resid(P, G, res, k, a, nullptr, nullptr);
             if (srcstage) sample_src(P, G, a, srcstage + (size_t)(k - 1) * G.S.n);
         }
@@ -1597,6 +1600,7 @@ static int el_sweep(prop_s *P, const Geometry &G, const float *res, const float 
     }
     // k = nt-1: the transposed step of a zero state is zero; the last residual sample
     WP_TRY(zero_fields(P, P->tmp + 9, 6));      // edge and face product sums
+    WP_TRY(zero_fields(P, P->tmp, 6));          // sigma of the zero state
     after(nt - 1);
     const int sf = (int)snap_fields(P);
     auto xs = [&](float *base, const float **out) {
@@ -2744,6 +2748,7 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
         WP_TRY(zero_fields(P, P->st, 9));
         WP_TRY(zero_fields(P, P->ast, 9));
         WP_TRY(zero_fields(P, P->tmp + 9, 6));     // edge and face product sums
+        WP_TRY(zero_fields(P, P->tmp, 6));         // sigma of the zero state
         return PROP_OK;
     };
     for (int i = 0; i < n; i++)
@@ -2850,14 +2855,9 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
         return PROP_OK;
     };
     // transposed step k = t - 1 with imaging at position pos: t -= 1, the
-    // pointwise kernel before, the three passes, the face products, the
-    // residual r^k
+    // three passes, the face products, the residual r^k
     auto adj = [&](int pos) -> int {
         k_tick(P0, tdev, -1);
-        WP_TRY(per_shot([&](int i) -> int {
-            el_adj_pre_launch(shots[i], shots[i]->ast, shots[i]->stream);
-            return PROP_OK;
-        }));
         WP_TRY(launch(1 + pos));
         WP_TRY(per_shot([&](int i) -> int {
             prop_s *P = shots[i];
@@ -2865,8 +2865,7 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
             xs(i, pos, x0);
             xs(i, pos + 1, x1);
             el_face2_launch(P, P->ast, x0, x1, P->stream);
-            float *const *a = P->ast;
-            sp_inject(P, &G[i].R, (const float *)tr[i].p, nt, 0, 1.f, 0, a[3], a[4], a[5], nullptr, nullptr, tdev);
+            sp_inject_t(P, &G[i].R, (const float *)tr[i].p, nt, 0, P->ast + 3, P->tmp, tdev);
             return PROP_OK;
         }));
         return PROP_OK;
@@ -2935,8 +2934,7 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
     // is zero; the last residual sample), then the segments, last first ----
     for (int i = 0; i < n; i++) {
         prop_s *P = shots[i];
-        float *const *a = P->ast;
-        sp_inject(P, &G[i].R, (const float *)tr[i].p, nt, nt - 1, 1.f, 0, a[3], a[4], a[5], nullptr, nullptr);
+        sp_inject_t(P, &G[i].R, (const float *)tr[i].p, nt, nt - 1, P->ast + 3, P->tmp);
     }
     for (int j = J - 1; j >= 0; j--) {
         const int n0 = j * K, E = std::min(n0 + K, nt - 1), len = E - n0;

@@ -72,7 +72,8 @@ __global__ void record_s_kernel(GridDev g, int n, const long long *__restrict__ 
                                 const float *__restrict__ f2, const float *__restrict__ lam,
                                 const float *__restrict__ mu, float nl, float scale, float *__restrict__ out)
 {
-    // nl = 3 (3D) or 2 (x-z plane, f2 == NULL): C of the unit diagonal is (nl lambda + 2 mu)
+    // nl = 3 (3D) or 2 (x-z plane, f2 == NULL): C of the unit diagonal is (nl lambda + 2 mu);
+    // nl = 0: the fields are t = g tbar itself
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float s = 0.f;
@@ -85,10 +86,33 @@ __global__ void record_s_kernel(GridDev g, int n, const long long *__restrict__ 
             const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY),
                       x = (int)(q / ((long long)g.PZ * g.NY));
             const float gn = g.tab[2 * x] * g.tab[2 * g.NX + 2 * y] * g.tab[2 * (g.NX + g.NY) + 2 * z];
-            s += wc * (f0[q] + f1[q] + (f2 ? f2[q] : 0.f)) / ((nl * lam[q] + 2.f * mu[q]) * gn);
+            s += wc * (f0[q] + f1[q] + (f2 ? f2[q] : 0.f)) / (nl > 0.f ? (nl * lam[q] + 2.f * mu[q]) * gn : gn);
         }
     }
     out[i] = scale * s;
+}
+
+// residual of the elastic transposed step in the form t = g tbar, sigma = C t:
+// d = g r into each diagonal component of t, (3 lambda + 2 mu) d into sigma's
+__global__ void inject_t_kernel(GridDev g, int ncell, const long long *__restrict__ cell, const int *__restrict__ ptr,
+                                const int *__restrict__ tr, const float *__restrict__ w,
+                                const float *__restrict__ traces, int nt, int t, const float *__restrict__ lam,
+                                const float *__restrict__ mu, float *t0, float *t1, float *t2, float *s0, float *s1,
+                                float *s2, const int *__restrict__ tdev)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= ncell) return;
+    if (tdev) t = *tdev;
+    const long long q = cell[j];
+    const int z = (int)(q % g.PZ), y = (int)((q / g.PZ) % g.NY), x = (int)(q / ((long long)g.PZ * g.NY));
+    const float gn = g.tab[2 * x] * g.tab[2 * g.NX + 2 * y] * g.tab[2 * (g.NX + g.NY) + 2 * z];
+    const float d = gn * inject_sum(ptr, tr, w, traces, nt, t, j), e = (3.f * lam[q] + 2.f * mu[q]) * d;
+    t0[q] += d;
+    t1[q] += d;
+    t2[q] += d;
+    s0[q] += e;
+    s1[q] += e;
+    s2[q] += e;
 }
 
 __global__ void transpose_kernel(const float *__restrict__ in, float *__restrict__ out, int n, int nt)
@@ -431,6 +455,24 @@ void sp_record_trace_s(prop_s *P, const SparseDev *S, const float *f0, const flo
     if (S->n <= 0) return;
     record_s_kernel<<<nblk(S->n), NB, 0, P->stream>>>(P->g, S->n, S->rec_idx, S->rec_w, f0, f1, f2, P->lam,
                                                       P->mu, f2 ? 3.f : 2.f, scale, out_col);
+    P->kern_launches++;
+}
+
+void sp_inject_t(prop_s *P, const SparseDev *S, const float *traces, int nt, int t, float *const *tt, float *const *sg,
+                 const int *tdev)
+{
+    if (S->ncell <= 0) return;
+    inject_t_kernel<<<nblk(S->ncell), NB, 0, P->stream>>>(P->g, S->ncell, S->cell, S->cell_ptr, S->ent_trace, S->ent_w,
+                                                          traces, nt, t, P->lam, P->mu, tt[0], tt[1], tt[2], sg[0],
+                                                          sg[1], sg[2], tdev);
+    P->kern_launches++;
+}
+
+void sp_record_trace_t(prop_s *P, const SparseDev *S, float *const *tt, float scale, float *out_col)
+{
+    if (S->n <= 0) return;
+    record_s_kernel<<<nblk(S->n), NB, 0, P->stream>>>(P->g, S->n, S->rec_idx, S->rec_w, tt[0], tt[1], tt[2], P->lam,
+                                                      P->mu, 0.f, scale, out_col);
     P->kern_launches++;
 }
 

@@ -48,8 +48,8 @@ namespace {
 struct F9 {
     float *f[9];
 };
-struct F5 {
-    float *f[5];
+struct F6 {
+    float *f[6];
 };
 
 
@@ -148,7 +148,7 @@ WP_DEV void v_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, 
 }
 
 template <int M, int ADJ>
-WP_DEV void v_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, const float *S, const ElCtx<M> &t,
+WP_DEV void v_plane(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, const float *S, const ElCtx<M> &t,
                     int x, float2 (&qxx)[2 * M], float2 (&qxy)[2 * M], float2 (&qxz)[2 * M])
 {
     using L = VL<M>;
@@ -225,7 +225,7 @@ WP_DEV void v_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
 
 // one tile (bx, by: z and y tile; bz: x chunk of xc planes)
 template <int M, int ADJ>
-WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, const VMaps &mp, int bx,
+WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, const VMaps &mp, int bx,
                           int by, int bz, int xc, int *err)
 {
     using L = VL<M>;
@@ -264,7 +264,7 @@ WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 
 
 template <int M, int ADJ>
 __global__ void __launch_bounds__(NTP, occ(M <= 4 ? 2 : 1))
-el_vpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ VMaps mp, const __grid_constant__ RecDev rec, int xc,
+el_vpass_tma(GridDev g, FDW w, F9 s, F6 o, const __grid_constant__ VMaps mp, const __grid_constant__ RecDev rec, int xc,
              int *err)
 {
     if (ADJ == 0 && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
@@ -276,13 +276,13 @@ el_vpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ VMaps mp, con
 // (s.f[0..2]) and
 //   MODE 0  tau <- g (tau + dt C S(v))                     (forward step)
 //   MODE 1  tbar <- t - dt S(w), t = g tbar, w = b_avg vbar  (stress half of
-//           the transposed step in the tbar form; t read, tbar written in
-//           s.f[3..8])
+//           the transposed step in the tbar form), and at once what the next
+//           step starts from: t <- g tbar (s.f[3..8]) and sigma = C t (o.f)
 //   MODE 2  imaging with the forward v^{k+1}: g_lambda += dt tr(t) tr(S v),
 //           g_mu += 2 dt sum_i t_ii S_ii, edge products dt t_c S_c
 //           (o.f = g_lambda, g_mu, xy, xz, yz products)
-// stage: [vx rect] [vy rect] [vz rect] (+ [mu +1 box, planes x, x+1] MODE 0)
-//        [t_xx .. t_yz (plane x)] (+ [lambda] MODE 0) (+ [g_lambda, g_mu]
+// stage: [vx rect] [vy rect] [vz rect] (+ [mu +1 box, planes x, x+1] MODE 0, 1)
+//        [t_xx .. t_yz (plane x)] (+ [lambda] MODE 0, 1) (+ [g_lambda, g_mu]
 //        MODE 2) [queue heads: vx (x+M-1), vy (x+M), vz (x+M)]
 // x-derivative queues: qvx[j] = v_x(x - M + j), qvy[j] = v_y(x - M + 1 + j),
 // qvz[j] = v_z(x - M + 1 + j).
@@ -290,10 +290,10 @@ el_vpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ VMaps mp, con
 template <int M, int MODE>
 struct TL {
     using B = BX<M>;
-    static constexpr int NP = MODE == 0 ? 2 : 0;           // +1 boxes
-    static constexpr int NI = 6 + (MODE == 0 ? 1 : 0) + (MODE == 2 ? 2 : 0) + 3;
+    static constexpr int NP = MODE != 2 ? 2 : 0;           // +1 boxes
+    static constexpr int NI = 6 + (MODE != 2 ? 1 : 2) + 3;
     static constexpr int OVX = 0, OVY = B::RS, OVZ = 2 * B::RS, OM0 = 3 * B::RS, OM1 = OM0 + B::PS,
-                         OT = 3 * B::RS + NP * B::PS, OL = OT + 6 * IS, OG = OL + (MODE == 0 ? IS : 0),
+                         OT = 3 * B::RS + NP * B::PS, OL = OT + 6 * IS, OG = OL + (MODE != 2 ? IS : 0),
                          OQ = OG + (MODE == 2 ? 2 * IS : 0), SZ = OQ + 3 * IS;
     static constexpr uint32_t BYTES = 4u * (3 * B::RR * B::RC + NP * B::PR * B::PC + NI * IS);
 };
@@ -311,7 +311,7 @@ WP_DEV void t_issue(const TMaps &mp, float *S, uint64_t *bar, int z0, int y0, in
     tma3(S + L::OVX, &mp.vx, z0 - B::MZ, y0 - M, x, bar);
     tma3(S + L::OVY, &mp.vy, z0 - B::MZ, y0 - M, x, bar);
     tma3(S + L::OVZ, &mp.vz, z0 - B::MZ, y0 - M, x, bar);
-    if (MODE == 0) {
+    if (MODE != 2) {
         tma3(S + L::OM0, &mp.mu, z0, y0, x, bar);
         tma3(S + L::OM1, &mp.mu, z0, y0, min(x + 1, NX - 1), bar);
         tma3(S + L::OL, &mp.lam, z0, y0, x, bar);
@@ -342,7 +342,7 @@ WP_DEV void t_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, 
 }
 
 template <int M, int MODE>
-WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, const float *S, const ElCtx<M> &t,
+WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, const float *S, const ElCtx<M> &t,
                     int x, float2 (&qvx)[2 * M], float2 (&qvy)[2 * M], float2 (&qvz)[2 * M])
 {
     using L = TL<M, MODE>;
@@ -383,7 +383,7 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
         const float2 t0 = lds2(T), t1 = lds2(T + IS), t2 = lds2(T + 2 * IS);
         const float2 t3 = lds2(T + 3 * IS), t4 = lds2(T + 4 * IS), t5 = lds2(T + 5 * IS);
         const unsigned q = x * (unsigned)g.NY * (unsigned)g.PZ + t.q0;
-        if (MODE == 0) {
+        if (MODE != 2) {
             const float *R0 = S + L::OM0, *R1 = S + L::OM1;
             const float2 m0 = lds2(R0 + ty * B::PC + c2), my = lds2(R0 + t.yb1 * B::PC + c2);
             const float2 mx = lds2(R1 + ty * B::PC + c2), mxy_ = lds2(R1 + t.yb1 * B::PC + c2);
@@ -404,19 +404,37 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
             const float myzb = 0.25f * (m0.y + my.y + m0z + myz);
             const float tra = exa + eya + eza, trb = exb + eyb + ezb;
             const float m2a = 2.f * m0.x, m2b = 2.f * m0.y;
-            st2(s.f[3], q, gn0 * (t0.x + c * (l.x * tra + m2a * exa)), gn1 * (t0.y + c * (l.y * trb + m2b * exb)));
-            st2(s.f[4], q, gn0 * (t1.x + c * (l.x * tra + m2a * eya)), gn1 * (t1.y + c * (l.y * trb + m2b * eyb)));
-            st2(s.f[5], q, gn0 * (t2.x + c * (l.x * tra + m2a * eza)), gn1 * (t2.y + c * (l.y * trb + m2b * ezb)));
-            st2(s.f[6], q, gxh * gyh * gzn0 * (t3.x + c * mxya * gxya), gxh * gyh * gzn1 * (t3.y + c * mxyb * gxyb));
-            st2(s.f[7], q, gxh * gyn * gzh0 * (t4.x + c * mxza * gxza), gxh * gyn * gzh1 * (t4.y + c * mxzb * gxzb));
-            st2(s.f[8], q, gxn * gyh * gzh0 * (t5.x + c * myza * gyza), gxn * gyh * gzh1 * (t5.y + c * myzb * gyzb));
-        } else if (MODE == 1) {
-            st2(s.f[3], q, t0.x - c * exa, t.two ? t0.y - c * exb : 0.f);
-            st2(s.f[4], q, t1.x - c * eya, t.two ? t1.y - c * eyb : 0.f);
-            st2(s.f[5], q, t2.x - c * eza, t.two ? t2.y - c * ezb : 0.f);
-            st2(s.f[6], q, t3.x - c * gxya, t.two ? t3.y - c * gxyb : 0.f);
-            st2(s.f[7], q, t4.x - c * gxza, t.two ? t4.y - c * gxzb : 0.f);
-            st2(s.f[8], q, t5.x - c * gyza, t.two ? t5.y - c * gyzb : 0.f);
+            const float gxy0 = gxh * gyh * gzn0, gxy1 = gxh * gyh * gzn1, gxz0 = gxh * gyn * gzh0;
+            const float gxz1 = gxh * gyn * gzh1, gyz0 = gxn * gyh * gzh0, gyz1 = gxn * gyh * gzh1;
+            if (MODE == 0) {
+                st2(s.f[3], q, gn0 * (t0.x + c * (l.x * tra + m2a * exa)), gn1 * (t0.y + c * (l.y * trb + m2b * exb)));
+                st2(s.f[4], q, gn0 * (t1.x + c * (l.x * tra + m2a * eya)), gn1 * (t1.y + c * (l.y * trb + m2b * eyb)));
+                st2(s.f[5], q, gn0 * (t2.x + c * (l.x * tra + m2a * eza)), gn1 * (t2.y + c * (l.y * trb + m2b * ezb)));
+                st2(s.f[6], q, gxy0 * (t3.x + c * mxya * gxya), gxy1 * (t3.y + c * mxyb * gxyb));
+                st2(s.f[7], q, gxz0 * (t4.x + c * mxza * gxza), gxz1 * (t4.y + c * mxzb * gxzb));
+                st2(s.f[8], q, gyz0 * (t5.x + c * myza * gyza), gyz1 * (t5.y + c * myzb * gyzb));
+            } else {
+                // lambda = mu = 0 in the row padding, so sigma is zero there by itself
+                const float a0 = gn0 * (t0.x - c * exa), b0 = t.two ? gn1 * (t0.y - c * exb) : 0.f;
+                const float a1 = gn0 * (t1.x - c * eya), b1 = t.two ? gn1 * (t1.y - c * eyb) : 0.f;
+                const float a2 = gn0 * (t2.x - c * eza), b2 = t.two ? gn1 * (t2.y - c * ezb) : 0.f;
+                const float a3 = gxy0 * (t3.x - c * gxya), b3 = t.two ? gxy1 * (t3.y - c * gxyb) : 0.f;
+                const float a4 = gxz0 * (t4.x - c * gxza), b4 = t.two ? gxz1 * (t4.y - c * gxzb) : 0.f;
+                const float a5 = gyz0 * (t5.x - c * gyza), b5 = t.two ? gyz1 * (t5.y - c * gyzb) : 0.f;
+                const float la = l.x * (a0 + a1 + a2), lb = l.y * (b0 + b1 + b2);
+                st2(s.f[3], q, a0, b0);
+                st2(s.f[4], q, a1, b1);
+                st2(s.f[5], q, a2, b2);
+                st2(s.f[6], q, a3, b3);
+                st2(s.f[7], q, a4, b4);
+                st2(s.f[8], q, a5, b5);
+                st2(o.f[0], q, la + m2a * a0, lb + m2b * b0);
+                st2(o.f[1], q, la + m2a * a1, lb + m2b * b1);
+                st2(o.f[2], q, la + m2a * a2, lb + m2b * b2);
+                st2(o.f[3], q, mxya * a3, mxyb * b3);
+                st2(o.f[4], q, mxza * a4, mxzb * b4);
+                st2(o.f[5], q, myza * a5, myzb * b5);
+            }
         } else {
             const float2 gl = lds2(S + L::OG + ii), gm = lds2(S + L::OG + IS + ii);
             st2(o.f[0], q, gl.x + c * (t0.x + t1.x + t2.x) * (exa + eya + eza),
@@ -441,7 +459,7 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, co
 }
 
 template <int M, int MODE>
-WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 &o, const TMaps &mp,
+WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, const TMaps &mp,
                           const InjDev *inj, int bx, int by, int bz, int xc, int *err)
 {
     using L = TL<M, MODE>;
@@ -486,7 +504,7 @@ WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F5 
 
 template <int M, int MODE>
 __global__ void __launch_bounds__(NTP, occ(M <= 4 ? 2 : 1))
-el_tpass_tma(GridDev g, FDW w, F9 s, F5 o, const __grid_constant__ TMaps mp, const __grid_constant__ InjDev inj, int xc,
+el_tpass_tma(GridDev g, FDW w, F9 s, F6 o, const __grid_constant__ TMaps mp, const __grid_constant__ InjDev inj, int xc,
              int *err)
 {
     el_tpass_body<M, MODE>(g, w, s, o, mp, &inj, blockIdx.x, blockIdx.y, blockIdx.z, xc, err);
@@ -499,7 +517,7 @@ struct ElShot {
     TMaps tm;
     GridDev g;
     F9 s;
-    F5 o;
+    F6 o;
     int xc;
     int *flag;
 };
@@ -1160,7 +1178,7 @@ dim3 el_grid(const prop_s *P)
 }
 
 template <int M, int ADJ>
-int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const VMaps &vm)
+int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F6 &o, const VMaps &vm)
 {
     const size_t sm = NSTAGE * VL<M>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(el_vpass_tma<M, ADJ>, sm);
@@ -1174,7 +1192,7 @@ int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const VMaps 
     return PROP_OK;
 }
 template <int M, int MODE>
-int launch_t(prop_s *P, const GridDev &g, const F9 &s, const F5 &o, const TMaps &tm)
+int launch_t(prop_s *P, const GridDev &g, const F9 &s, const F6 &o, const TMaps &tm)
 {
     const size_t sm = NSTAGE * TL<M, MODE>::SZ * sizeof(float) + 64;
     static const bool attr = set_smem(el_tpass_tma<M, MODE>, sm);
@@ -1192,7 +1210,7 @@ int el_launch(prop_s *P, float *const *S, float dt)
     g.dt = dt;
     F9 s;                                      // the new velocities and, in place, the stresses
     for (int i = 0; i < 9; i++) s.f[i] = i < 3 && P->out[i] ? P->out[i] : S[i];
-    const F5 o{};
+    const F6 o{};
     VMaps vm;
     TMaps tm;
     if (!vmaps<M>(P, S, S + 3, &vm) || !tmaps<M>(P, s.f, S + 3, &tm))
@@ -1205,7 +1223,7 @@ int el_launch(prop_s *P, float *const *S, float dt)
 // on entry S[3..8] = t = g tbar and sig[0..5] = C t; S[0..2] = vbar.
 //   vbar <- g (vbar - dt Dtau(sig)),  w = b_avg vbar   (w[0..2])
 //   g_lambda, g_mu, edge products from t and S(v^{k+1})
-//   tbar <- t - dt S(w)
+//   tbar <- t - dt S(w); t, sig <- g tbar, C t of the next step
 template <int M>
 int el_adj_grad(prop_s *P, float *const *S, float *const *sig, float *const *w, const float *const *v1,
                 float *const *gr, float *const *ep)
@@ -1227,10 +1245,11 @@ int el_adj_grad(prop_s *P, float *const *S, float *const *sig, float *const *w, 
         sg.f[3 + i] = S[3 + i];
         st.f[3 + i] = S[3 + i];
     }
-    const F5 ow{{w[0], w[1], w[2], nullptr, nullptr}}, og{{gr[0], gr[1], ep[0], ep[1], ep[2]}}, none{};
+    const F6 ow{{w[0], w[1], w[2]}}, og{{gr[0], gr[1], ep[0], ep[1], ep[2]}},
+        os{{sig[0], sig[1], sig[2], sig[3], sig[4], sig[5]}};
     WP_TRY((launch_v<M, 1>(P, g, sv, ow, vm)));
     WP_TRY((launch_t<M, 2>(P, g, sg, og, tg)));
-    return launch_t<M, 1>(P, g, st, none, tt);
+    return launch_t<M, 1>(P, g, st, os, tt);
 }
 
 template <int M, int ADJ, int GRAD>
@@ -2079,7 +2098,7 @@ static int el_fill(const ElBatchReq *req, int n, ElShot *H, std::string *err)
             e.g = P->g;
             e.g.dt = req[i].sign * P->g.dt;
             for (int k = 0; k < 9; k++) e.s.f[k] = S[k];
-            e.o = F5{};
+            e.o = F6{};
             ok = vmaps<M>(P, S, S + 3, &e.vm) && tmaps<M>(P, S, S + 3, &e.tm);
             e.xc = P->xchunk;
             e.flag = P->flag;
@@ -2093,7 +2112,7 @@ static int el_fill(const ElBatchReq *req, int n, ElShot *H, std::string *err)
                 e->g = P->g;
                 e->xc = P->xchunk;
                 e->flag = P->flag;
-                e->o = F5{};
+                e->o = F6{};
             }
             for (int k = 0; k < 3; k++) {
                 ev.s.f[k] = S[k];
@@ -2106,7 +2125,8 @@ static int el_fill(const ElBatchReq *req, int n, ElShot *H, std::string *err)
                 e2.s.f[3 + k] = S[3 + k];
                 e1.s.f[3 + k] = S[3 + k];
             }
-            e2.o = F5{{req[i].g[0], req[i].g[1], ep[0], ep[1], ep[2]}};
+            e2.o = F6{{req[i].g[0], req[i].g[1], ep[0], ep[1], ep[2]}};
+            for (int k = 0; k < 6; k++) e1.o.f[k] = sig[k];
             ok = vmaps<M>(P, S, sig, &ev.vm) && tmaps<M>(P, v1, S + 3, &e2.tm) && tmaps<M>(P, w, S + 3, &e1.tm) &&
                  map_of(P, req[i].g[0], FZ, FY, &e2.tm.gl) && map_of(P, req[i].g[1], FZ, FY, &e2.tm.gm);
         }
@@ -2174,7 +2194,6 @@ static int el_batch_launch(TtiBatch *b, const ElBatchReq *req, int n, cudaStream
         static const bool attr = set_smem(el_vpass_batch<M, 1>, sv) && set_smem(el_tpass_batch<M, 2>, s2) &&
                                  set_smem(el_tpass_batch<M, 1>, s1);
         (void)attr;
-        for (int i = 0; i < n; i++) el_adj_pre_launch(req[i].P, req[i].S, st);
         el_vpass_batch<M, 1><<<nt, blk, sv, st>>>(D, b->dtiles, w);
         el_tpass_batch<M, 2><<<nt, blk, s2, st>>>(D + n, b->dtiles, w);
         el_tpass_batch<M, 1><<<nt, blk, s1, st>>>(D + 2 * n, b->dtiles, w);
