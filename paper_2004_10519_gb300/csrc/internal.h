@@ -19,13 +19,14 @@ constexpr int INJ_MAX = 16;  // source cells that a pass injects itself; more go
 // Computational grid as seen by the kernels.  Index (x,y,z) -> (x*NY + y)*PZ + z.
 struct GridDev {
     int NX, NY, NZ;          // computational grid
-    int PZ;                  // row pitch in floats (>= NZ): a multiple of 4 where the TMA-fed passes run
     int nbl, px, py, pz;     // absorbing width, physical grid
     int nby;                 // absorbing width on the y faces (0 in 2D)
     long long N;             // elements of a field, NX*NY*PZ
     float h, ih, dt;         // spacing, 1/h, time step
     float sig0;              // TTI damping: sigma(d) = sig0 * (d/L)^2 per axis [1/s]
     float cer;               // elastic Cerjan coefficient per cell (0.015)
+    int PZ;                  // row pitch in floats (>= NZ): a multiple of 4 where the TMA-fed passes run (in the
+                             // struct's hole: 8 bytes more of it cost the acoustic pass 6 registers)
     // per-axis absorbing-layer tables (device):
     //   TTI:     sigma_x[NX], sigma_y[NY], sigma_z[NZ]  (sigma = sum of the three)
     //   elastic: taper_x[2 NX], taper_y[2 NY], taper_z[2 NZ]; entry 2i is the
@@ -83,7 +84,7 @@ struct prop_s {
     FDW w{};
     int M = 0;
     cudaStream_t stream = nullptr;
-    int dev = 0;             // device of the handle
+    int dev = 0, sms = 152;  // device of the handle and its SMs
     bool broken = false;
     std::string err;
     float vmax = 0.f;        // max model velocity used for the CFL rule
@@ -217,8 +218,8 @@ void tti_axis_to_angles(prop_s *P, float *const *a);
 // TMA passes of a transposed elastic step with imaging: on entry S[3..8] hold
 // t = g tbar and sig[0..5] = C t; updates vbar (S[0..2]), writes b_avg vbar to
 // w[0..2], accumulates g_lambda, g_mu (gr[0], gr[1]) and the edge products
-// ep[0..2] with the strain of v1 (forward velocities at k+1), then
-// tbar = t - dt S(w) into S[3..8]
+// ep[0..2] with the strain of v1 (forward velocities at k+1), then with
+// tbar = t - dt S(w) leaves the next step's t = g tbar in S[3..8] and C t in sig
 int el_adj_grad_tma(prop_s *P, float *const *S, float *const *sig, float *const *w, const float *const *v1,
                     float *const *gr, float *const *ep);
 int tti_launch_tma(prop_s *P, float *const *S, bool adjoint, const float *img_p,
