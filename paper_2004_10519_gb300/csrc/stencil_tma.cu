@@ -11,7 +11,7 @@
 // finite-difference operators.  Every other per-plane input (the thread's
 // own values, parameters, the new head of each x-derivative queue M planes
 // ahead) comes through the same ring as an interior box.  The ring is a
-// producer/consumer pipeline on mbarriers (RingN in tma.cuh): a dedicated
+// producer/consumer pipeline on mbarriers (Ring in tma.cuh): a dedicated
 // producer warp refills a stage as soon as every consumer warp has released
 // it, and no CTA-wide barrier is taken per plane (the acoustic pass uses a
 // 32 x 32 tile, two rows per thread).
@@ -230,8 +230,9 @@ WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 
 {
     using L = VL<M>;
     constexpr int Q = 2 * M;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + NSTAGE * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, warp = (ty * TZ2 + tz) >> 5, lane = (ty * TZ2 + tz) & 31;
     const bool lead = warp == 0 && lane == 0;
     const int z0 = bx * FZ, y0 = by * FY;
@@ -240,7 +241,7 @@ WP_DEV void el_vpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 
     Ring R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -464,8 +465,9 @@ WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 
 {
     using L = TL<M, MODE>;
     constexpr int Q = 2 * M;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + NSTAGE * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, warp = (ty * TZ2 + tz) >> 5, lane = (ty * TZ2 + tz) & 31;
     const bool lead = warp == 0 && lane == 0;
     const int z0 = bx * FZ, y0 = by * FY;
@@ -474,7 +476,7 @@ WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 
     Ring R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -578,8 +580,9 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
     using L = RL<M>;
     using B = BX<M>;
     constexpr int Q = 2 * M + 1;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + L::NS * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, lane = (ty * TZ2 + tz) & 31;
     const bool lead = ty == 0 && tz == 0;
     const int z0 = bx * FZ, y0 = by * FY;
@@ -596,10 +599,10 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
         tma3(S + L::ON, &mp.nx, z0, y0, x, bar);
         tma3(S + L::ON + IS, &mp.ny, z0, y0, x, bar);
     };
-    RingN<L::NS> R(bars);
+    Ring R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -765,8 +768,9 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
     using L = UL<M, ADJ, GRAD>;
     using B = BX<M>;
     constexpr int Q = 2 * M + 1;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + NSTAGE * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, warp = (ty * TZ2 + tz) >> 5, lane = (ty * TZ2 + tz) & 31;
     const bool lead = warp == 0 && lane == 0;
     const int z0 = bx * FZ, y0 = by * FY;
@@ -804,7 +808,7 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
     Ring R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -1016,8 +1020,9 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
     if (!GRAD && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
     using L = AL<M, GRAD>;
     constexpr int Q = 2 * M + 1;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + L::NS * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, lane = (ty * TZ2 + tz) & 31;
     const bool lead = ty == 0 && tz == 0;
     const int z0 = blockIdx.x * FZ, y0 = blockIdx.y * AFY;
@@ -1037,10 +1042,10 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
             tma3(I + L::GG * AIS, &mp.g, z0, y0, x, bar);
         }
     };
-    RingN<L::NS> R(bars);
+    RingN<(M > 4 ? L::NS : 0)> R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -1180,11 +1185,11 @@ dim3 el_grid(const prop_s *P)
 template <int M, int ADJ>
 int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F6 &o, const VMaps &vm)
 {
-    const size_t sm = NSTAGE * VL<M>::SZ * sizeof(float) + 64;
-    static const bool attr = set_smem(el_vpass_tma<M, ADJ>, sm);
+    static const bool attr = set_smem(el_vpass_tma<M, ADJ>, SMEM_MAX);
     (void)attr;
     dim3 grd = el_grid(P), blk(TZ2, FY + 2, 1);
     const RecDev rec = ADJ ? RecDev{} : P->rec;
+    const size_t sm = ring_smem(P, grd, occ(M <= 4 ? 2 : 1), VL<M>::SZ, NSTAGE);
     grd.z += receiver_layers(rec, grd, blk);
     launch_pass(el_vpass_tma<M, ADJ>, grd, blk, sm, P->stream, g, P->w, s, o, vm, rec, P->xchunk, P->flag);
     P->kern_launches++;
@@ -1194,8 +1199,8 @@ int launch_v(prop_s *P, const GridDev &g, const F9 &s, const F6 &o, const VMaps 
 template <int M, int MODE>
 int launch_t(prop_s *P, const GridDev &g, const F9 &s, const F6 &o, const TMaps &tm)
 {
-    const size_t sm = NSTAGE * TL<M, MODE>::SZ * sizeof(float) + 64;
-    static const bool attr = set_smem(el_tpass_tma<M, MODE>, sm);
+    const size_t sm = ring_smem(P, el_grid(P), occ(M <= 4 ? 2 : 1), TL<M, MODE>::SZ, NSTAGE);
+    static const bool attr = set_smem(el_tpass_tma<M, MODE>, SMEM_MAX);
     (void)attr;
     launch_pass(el_tpass_tma<M, MODE>, el_grid(P), dim3(TZ2, FY + 2, 1), sm, P->stream, g, P->w, s, o, tm, MODE == 0 ? P->inj : InjDev{}, P->xchunk, P->flag);
     P->kern_launches++;
@@ -1280,9 +1285,9 @@ int tti_launch(prop_s *P, float *const *S, const float *up, const float *ur, flo
         ok = ok && map_of(P, up, FZ, FY, &um.up) && map_of(P, ur, FZ, FY, &um.ur) &&
              map_of(P, grad, FZ, FY, &um.g);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-    const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64,
-                 s2 = NSTAGE * UL<M, ADJ, GRAD>::SZ * sizeof(float) + 64;
-    static const bool attr = set_smem(tti_rot_tma<M>, s1) && set_smem(tti_upd_tma<M, ADJ, GRAD>, s2);
+    const size_t s1 = ring_smem(P, grd, occ(2), RL<M>::SZ, RL<M>::NS),
+                 s2 = ring_smem(P, grd, occ(2), UL<M, ADJ, GRAD>::SZ, NSTAGE);
+    static const bool attr = set_smem(tti_rot_tma<M>, SMEM_MAX) && set_smem(tti_upd_tma<M, ADJ, GRAD>, SMEM_MAX);
     (void)attr;
     const RecDev rec = ADJ ? RecDev{} : P->rec;
     const dim3 grd1(grd.x, grd.y, grd.z + receiver_layers(rec, grd, blk));
@@ -1376,8 +1381,8 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
               map_of(P, lp, FZ, FY, &um.pc) && map_of(P, lr, FZ, FY, &um.rc) &&
               map_of(P, P->c2, FZ, FY, &um.d) && map_of(P, ge, FZ, FY, &um.up) && map_of(P, gd, FZ, FY, &um.ur);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-    const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * UL<M, 2, 0>::SZ * sizeof(float) + 64;
-    static const bool attr = set_smem(tti_rot_tma<M>, s1) && set_smem(tti_upd_tma<M, 2, 0>, s2);
+    const size_t s1 = ring_smem(P, grd, occ(2), RL<M>::SZ, RL<M>::NS), s2 = ring_smem(P, grd, occ(2), UL<M, 2, 0>::SZ, NSTAGE);
+    static const bool attr = set_smem(tti_rot_tma<M>, SMEM_MAX) && set_smem(tti_upd_tma<M, 2, 0>, SMEM_MAX);
     (void)attr;
     launch_pass(tti_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
                                                RecDev{}, xc, P->flag);
@@ -1390,7 +1395,7 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
              map_of(P, t[6], FZ, FY, &rz.qp) && map_of(P, t[7], FZ, FY, &rz.qr) && (rz.nx = rm.nx, true) &&
              (rz.ny = rm.ny, true);
         if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-        static const bool attr_raw = set_smem(tti_rot_tma<M, 1>, s1);
+        static const bool attr_raw = set_smem(tti_rot_tma<M, 1>, SMEM_MAX);
         (void)attr_raw;
         launch_pass(tti_rot_tma<M, 1>, grd, blk, s1, P->stream, g, P->w, t[6], t[7], rz, t[0], t[1], t[2], t[3], t[4], t[5],
                                                        F3{}, RecDev{}, xc, P->flag);
@@ -1433,8 +1438,9 @@ int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
               map_of(P, P->acw, FZ, AFY, &am.w) && map_of(P, S[1], FZ, AFY, &am.u0);
     if (GRAD) ok = ok && map_of(P, uf, FZ, AFY, &am.uf) && map_of(P, grad, FZ, AFY, &am.g);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-    const size_t sb = AL<M, GRAD>::NS * AL<M, GRAD>::SZ * sizeof(float) + 64;
-    static const bool attr = set_smem(acu_tma<M, GRAD>, sb);
+    const size_t sb = M > 4 ? ring_bytes(AL<M, GRAD>::NS, AL<M, GRAD>::SZ)
+                            : ring_smem(P, grd, 2, AL<M, GRAD>::SZ, AL<M, GRAD>::NS);
+    static const bool attr = set_smem(acu_tma<M, GRAD>, SMEM_MAX);
     (void)attr;
     const RecDev rec = GRAD ? RecDev{} : P->rec;
     grd.z += receiver_layers(rec, grd, blk);
@@ -1481,7 +1487,7 @@ int raw_half(prop_s *P, const float *p, const float *r, float *const *dp, float 
                     map_of(P, p, FZ, FY, &rm.qp) && map_of(P, r, FZ, FY, &rm.qr) &&
                     map_of(P, P->nrm[0], FZ, FY, &rm.nx) && map_of(P, P->nrm[1], FZ, FY, &rm.ny);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-    const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64;
+    const size_t s1 = ring_bytes(RL<M>::NS, RL<M>::SZ);
     static const bool attr = set_smem(tti_rot_tma<M, 2>, s1);
     (void)attr;
     launch_pass(tti_rot_tma<M, 2>, grd, blk, s1, P->stream, g, P->w, p, r, rm, dp[0], dp[1], dp[2], dr[0], dr[1], dr[2],
@@ -1637,7 +1643,7 @@ namespace {
 template <int M>
 size_t smem_need(int kind)
 {
-    auto b = [](int floats) { return (size_t)floats * sizeof(float) + 64; };
+    auto b = [](int floats) { return ring_bytes(1, floats); };
     if (kind == PROP_ELASTIC)
         return std::max({b(NSTAGE * VL<M>::SZ), b(NSTAGE * TL<M, 0>::SZ), b(NSTAGE * TL<M, 1>::SZ),
                          b(NSTAGE * TL<M, 2>::SZ)});
@@ -1867,8 +1873,8 @@ int tti_batch_launch(TtiBatch *b, const TtiBatchReq *req, int n, cudaStream_t st
                     "batched TTI step: shot table copy"))
         return rc;
     if (int rc = ck(cudaEventRecord(b->copied[slot], st), "batched TTI step: event")) return rc;
-    const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64,
-                 s2 = NSTAGE * UL<M, ADJ, GRAD>::SZ * sizeof(float) + 64;
+    const size_t s1 = ring_bytes(RL<M>::NS, RL<M>::SZ),
+                 s2 = ring_bytes(NSTAGE, UL<M, ADJ, GRAD>::SZ);
     static const bool attr = set_smem(tti_rot_batch<M>, s1) && set_smem(tti_upd_batch<M, ADJ, GRAD>, s2);
     (void)attr;
     const unsigned nt = (unsigned)b->htiles.size();
@@ -1994,8 +2000,8 @@ int tti_batch_fix(TtiBatch *b, const TtiBatchReq *req, int n, int slot, cudaStre
 template <int M, int ADJ, int GRAD>
 static int tti_batch_run_fixed(TtiBatch *b, int slot, cudaStream_t st)
 {
-    const size_t s1 = RL<M>::NS * RL<M>::SZ * sizeof(float) + 64,
-                 s2 = NSTAGE * UL<M, ADJ, GRAD>::SZ * sizeof(float) + 64;
+    const size_t s1 = ring_bytes(RL<M>::NS, RL<M>::SZ),
+                 s2 = ring_bytes(NSTAGE, UL<M, ADJ, GRAD>::SZ);
     static const bool attr = set_smem(tti_rot_batch<M>, s1) && set_smem(tti_upd_batch<M, ADJ, GRAD>, s2);
     (void)attr;
     const unsigned nt = (unsigned)b->htiles.size();
@@ -2183,14 +2189,14 @@ static int el_batch_launch(TtiBatch *b, const ElBatchReq *req, int n, cudaStream
     const ElShot *D = reinterpret_cast<const ElShot *>(b->del);
     const FDW &w = req[0].P->w;
     if (mode == 0) {
-        const size_t sv = NSTAGE * VL<M>::SZ * sizeof(float) + 64, stt = NSTAGE * TL<M, 0>::SZ * sizeof(float) + 64;
+        const size_t sv = ring_bytes(NSTAGE, VL<M>::SZ), stt = ring_bytes(NSTAGE, TL<M, 0>::SZ);
         static const bool attr = set_smem(el_vpass_batch<M, 0>, sv) && set_smem(el_tpass_batch<M, 0>, stt);
         (void)attr;
         el_vpass_batch<M, 0><<<nt, blk, sv, st>>>(D, b->dtiles, w);
         el_tpass_batch<M, 0><<<nt, blk, stt, st>>>(D, b->dtiles, w);
     } else {
-        const size_t sv = NSTAGE * VL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * TL<M, 2>::SZ * sizeof(float) + 64,
-                     s1 = NSTAGE * TL<M, 1>::SZ * sizeof(float) + 64;
+        const size_t sv = ring_bytes(NSTAGE, VL<M>::SZ), s2 = ring_bytes(NSTAGE, TL<M, 2>::SZ),
+                     s1 = ring_bytes(NSTAGE, TL<M, 1>::SZ);
         static const bool attr = set_smem(el_vpass_batch<M, 1>, sv) && set_smem(el_tpass_batch<M, 2>, s2) &&
                                  set_smem(el_tpass_batch<M, 1>, s1);
         (void)attr;
@@ -2285,7 +2291,7 @@ static int el_batch_run_fixed(TtiBatch *b, int slot, cudaStream_t st)
     const ElShot *D = b->elfixed[slot];
     const int n = b->fixed_n;
     if (b->elfixed_mode[slot] == 0) {
-        const size_t sv = NSTAGE * VL<M>::SZ * sizeof(float) + 64, stt = NSTAGE * TL<M, 0>::SZ * sizeof(float) + 64;
+        const size_t sv = ring_bytes(NSTAGE, VL<M>::SZ), stt = ring_bytes(NSTAGE, TL<M, 0>::SZ);
         static const bool attr = set_smem(el_vpass_batch<M, 0>, sv) && set_smem(el_tpass_batch<M, 0>, stt);
         (void)attr;
         el_vpass_batch<M, 0><<<nt, blk, sv, st>>>(D, b->dtiles, b->w);
@@ -2293,8 +2299,8 @@ static int el_batch_run_fixed(TtiBatch *b, int slot, cudaStream_t st)
     } else {
         // the three passes only: the pointwise kernels before and after are
         // the caller's (per shot)
-        const size_t sv = NSTAGE * VL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * TL<M, 2>::SZ * sizeof(float) + 64,
-                     s1 = NSTAGE * TL<M, 1>::SZ * sizeof(float) + 64;
+        const size_t sv = ring_bytes(NSTAGE, VL<M>::SZ), s2 = ring_bytes(NSTAGE, TL<M, 2>::SZ),
+                     s1 = ring_bytes(NSTAGE, TL<M, 1>::SZ);
         static const bool attr = set_smem(el_vpass_batch<M, 1>, sv) && set_smem(el_tpass_batch<M, 2>, s2) &&
                                  set_smem(el_tpass_batch<M, 1>, s1);
         (void)attr;

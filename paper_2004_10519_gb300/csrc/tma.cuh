@@ -13,6 +13,7 @@
 #include "tile.cuh"
 
 #include <cuda.h>
+#include <algorithm>
 #include <cstdlib>
 #include <mutex>
 
@@ -99,10 +100,9 @@ WP_DEV void mbar_arrive(uint64_t *bar)
 }
 // producer after an abort: wait (bounded) for the stages of iterations
 // [a, b] that may still be in flight, so no copy lands after the CTA exits
-template <int NS = NSTAGE>
-WP_DEV void drain(uint64_t *full, int a, int b)
+WP_DEV void drain(uint64_t *full, int ns, int a, int b)
 {
-    for (int j = a < 0 ? 0 : a; j <= b; j++) mbar_wait(&full[j % NS], (uint32_t)((j / NS) & 1));
+    for (int j = a < 0 ? 0 : a; j <= b; j++) mbar_wait(&full[j % ns], (uint32_t)((j / ns) & 1));
 }
 
 // 8-byte accesses (z even, row pitch even: always aligned)
@@ -254,50 +254,91 @@ WP_DEV void own_sources(const InjDev &I, unsigned q0, int xa, int xb, F f)
 // Producer/consumer plane ring.  full[s] completes when the copies of a
 // stage have landed (one arrive with the byte count + the TMA bytes);
 // empty[s] when every consumer warp has finished reading it (one arrive per
-// warp).  A dedicated producer warp (its lane 0) keeps NS planes in
+// warp).  A dedicated producer warp (its lane 0) keeps ns planes in
 // flight: it refills a stage as soon as it is released, so consumers never
 // wait for each other.  All waits are bounded; a warp that gives up reports
 // bit 2 and leaves, and the producer drains its copies in flight first.
 constexpr int NWARP = NT2 / 32;
 
-template <int NS = NSTAGE>
+// Stages of the ring: as many as the launch's dynamic shared memory holds behind
+// the barriers (8 full, 8 empty) and the number of stages, which the consumers
+// read there once a plane rather than hold in a register.
+constexpr int MAX_STAGES = 8, BAR_BYTES = 16 * MAX_STAGES + 128;
+// dynamic shared memory per CTA (1 KB below the opt-in limit, for static variables) and per SM
+constexpr size_t SMEM_MAX = 226 * 1024, SMEM_SM = 228 * 1024;
+constexpr size_t ring_bytes(int ns, int stage) { return (size_t)ns * stage * sizeof(float) + BAR_BYTES; }
+WP_DEV int ring_stages(int stage)
+{
+    unsigned dyn;
+    asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+    return (int)((dyn - BAR_BYTES) / (unsigned)(stage * sizeof(float)));
+}
+// Dynamic shared memory of a pass of `ctas` CTAs of which `occ` fit an SM: at least
+// `least` stages, and where the grid leaves an SM fewer CTAs than fit it, the
+// memory of the missing ones as further stages (up to the planes of a chunk).  A
+// plane's copies take about three times as long as its arithmetic, so three planes
+// in flight keep up when two CTAs or more share an SM, but not when one is alone.
+// TTI so 8, 84^3 (99 CTAs), 3 and 4 stages -> 7 and 8: 19.1 -> 17.5 us per step.
+inline size_t ring_smem(const prop_s *P, dim3 grd, int occ, int stage, int least)
+{
+    const long long ctas = (long long)grd.x * grd.y * grd.z;
+    const int res = (int)std::min<long long>(occ, std::max<long long>(1, (ctas + P->sms - 1) / P->sms));
+    int ns = least;
+    if (res < occ) {
+        const size_t room = std::min(SMEM_MAX, SMEM_SM / res - 1024);      // 1 KB per CTA is the system's
+        ns = (int)std::min<size_t>({(size_t)MAX_STAGES, (size_t)P->xchunk, (room - BAR_BYTES) / (stage * sizeof(float))});
+    }
+    return ring_bytes(std::max(ns, least), stage);
+}
+
+// NS > 0: that many stages, a constant (for a pass without a register to spare).
+template <int NS = 0>
 struct RingN {
-    uint64_t *full, *empty;
+    uint64_t *full;
     int st = 0;
     uint32_t ph = 0;
-    WP_DEV explicit RingN(uint64_t *bars) : full(bars), empty(bars + NS) {}
-    WP_DEV void init()
+    WP_DEV explicit RingN(uint64_t *bars) : full(bars) {}
+    WP_DEV uint64_t *empty(int s) { return full + MAX_STAGES + s; }
+    WP_DEV int stages() { return NS ? NS : *reinterpret_cast<const volatile int *>(full + 2 * MAX_STAGES); }
+    WP_DEV void init(int ns)
     {
-        for (int i = 0; i < NS; i++) {
+        *reinterpret_cast<volatile int *>(full + 2 * MAX_STAGES) = ns;
+        for (int i = 0; i < ns; i++) {
             mbar_init(&full[i], 1);
-            mbar_init(&empty[i], NWARP);
+            mbar_init(empty(i), NWARP);
         }
         fence_init();
     }
-    // producer (lane 0 of the producer warp): plane xa + it into stage it % NS
+    // producer (lane 0 of the producer warp): plane xa + it into stage it % ns
     template <class F>
     WP_DEV void produce(int xa, int nit, F issue, int *err)
     {
+        const int ns = stages();
+        int s = 0;
+        uint32_t lap = 1;                    // parity of the release of the lap before
         for (int it = 0; it < nit; it++) {
-            const int s = it % NS;
-            if (it >= NS && !mbar_wait(&empty[s], (uint32_t)(((it / NS) - 1) & 1))) {
+            if (it >= ns && !mbar_wait(empty(s), lap)) {
                 atomicOr(err, 2);
-                drain<NS>(full, it - NS, it - 1);
+                drain(full, ns, it - ns, it - 1);
                 return;
             }
             issue(xa + it, s);
+            if (++s == ns) {
+                s = 0;
+                lap ^= 1u;
+            }
         }
         // stay until the last copies have landed (bounded), so none can
         // arrive after the CTA has exited even if the consumers gave up
-        drain<NS>(full, nit - NS, nit - 1);
+        drain(full, ns, nit - ns, nit - 1);
     }
     WP_DEV bool wait_full() { return mbar_wait(&full[st], ph); }
     // end of iteration: this warp is done with the stage
     WP_DEV void release(int lane)
     {
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[st]);
-        if (++st == NS) {
+        if (lane == 0) mbar_arrive(empty(st));
+        if (++st == stages()) {
             st = 0;
             ph ^= 1u;
         }

@@ -50,8 +50,9 @@ tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__res
     using L = SRL<M>;
     using B = BX<M>;
     constexpr int Q = 2 * M + 1;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + NSTAGE * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, lane = (ty * TZ2 + tz) & 31;
     const bool lead = ty == 0 && tz == 0;
     const int z0 = blockIdx.x * FZ, y0 = blockIdx.y * FY;
@@ -72,7 +73,7 @@ tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__res
     Ring R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -283,8 +284,9 @@ tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float
     using L = SUL<M, ADJ, GRAD>;
     using B = BX<M>;
     constexpr int Q = 2 * M + 1;
-    extern __shared__ __align__(128) float sm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + NSTAGE * L::SZ);   // after the ring
+    extern __shared__ __align__(128) float dsm[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(dsm);
+    float *sm = dsm + BAR_BYTES / sizeof(float);                           // the ring
     const int tz = threadIdx.x, ty = threadIdx.y, lane = (ty * TZ2 + tz) & 31;
     const bool lead = ty == 0 && tz == 0;
     const int z0 = blockIdx.x * FZ, y0 = blockIdx.y * FY;
@@ -324,7 +326,7 @@ tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float
     Ring R(bars);
     pass_begins();
     if (lead) {
-        R.init();
+        R.init(ring_stages(L::SZ));
         ck_begin(g.N, err);
     }
     __syncthreads();
@@ -456,7 +458,7 @@ int sp_launch(prop_s *P, float *const *S, const float *up, const float *ur, floa
     if (GRAD)
         ok = ok && map_of(P, up, FZ, FY, &um.up) && map_of(P, ur, FZ, FY, &um.ur) && map_of(P, grad, FZ, FY, &um.g);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-    const size_t s1 = NSTAGE * SRL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * SUL<M, ADJ, GRAD>::SZ * sizeof(float) + 64;
+    const size_t s1 = ring_bytes(NSTAGE, SRL<M>::SZ), s2 = ring_bytes(NSTAGE, SUL<M, ADJ, GRAD>::SZ);
     static const bool attr = set_smem(tti_sp_rot_tma<M>, s1) && set_smem(tti_sp_upd_tma<M, ADJ, GRAD>, s2);
     (void)attr;
     launch_pass(tti_sp_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, rp_, rr_, rm, o, xc, P->flag);
@@ -558,7 +560,7 @@ int sp_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp,
     ok = ok && map_of(P, lp, FZ, FY, &um.pc) && map_of(P, lr, FZ, FY, &um.rc) && map_of(P, P->c2, FZ, FY, &um.d) &&
          map_of(P, ge, FZ, FY, &um.up) && map_of(P, gd, FZ, FY, &um.ur);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
-    const size_t s1 = NSTAGE * SRL<M>::SZ * sizeof(float) + 64, s2 = NSTAGE * SUL<M, 2, 0>::SZ * sizeof(float) + 64;
+    const size_t s1 = ring_bytes(NSTAGE, SRL<M>::SZ), s2 = ring_bytes(NSTAGE, SUL<M, 2, 0>::SZ);
     static const bool attr = set_smem(tti_sp_rot_tma<M>, s1) && set_smem(tti_sp_upd_tma<M, 2, 0>, s2);
     (void)attr;
     launch_pass(tti_sp_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, o, xc, P->flag);
