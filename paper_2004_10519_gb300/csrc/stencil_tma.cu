@@ -549,7 +549,8 @@ el_tpass_batch(const ElShot *__restrict__ shots, const int4 *__restrict__ tiles,
 // also the products of the staggered first derivatives at the half points,
 // h_i = (D+_i p)(D+_i r), D+_i f(q + 1/2) = sum_k b_k (f(q + k e_i) -
 // f(q - (k - 1) e_i)) / h, zero outside the grid (staggered-pair tilt/azimuth
-// imaging with p = zeta_p, r = u_p or p = zeta_r, r = u_r)
+// imaging with p = zeta_p, r = u_p or p = zeta_r, r = u_r).  MODE 3: e, f and also
+// D p, D r (hh): both that the imaging of a forward level needs, in one pass
 // stage: [p rect] [r rect] [queue heads p, r (x+M)] [n_x, n_y (plane x)]
 // ---------------------------------------------------------------------------
 template <int M>
@@ -565,18 +566,14 @@ struct RMaps {
 };
 
 // one tile (bx, by: 32 z x FY y columns; bz: x chunk of xc planes)
-struct F3 {
-    float *f[3];
-};
-
 template <int M, int MODE>
 WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict__ p,
                          const float *__restrict__ r, const RMaps &mp, float *__restrict__ ex,
                          float *__restrict__ ey, float *__restrict__ ez, float *__restrict__ fx,
-                         float *__restrict__ fy, float *__restrict__ fz, const F3 &hh, int bx, int by, int bz,
+                         float *__restrict__ fy, float *__restrict__ fz, const F6 &hh, int bx, int by, int bz,
                          int xc, int *err)
 {
-    constexpr bool RAW = MODE != 0, HALF = MODE == 2;
+    constexpr bool RAW = MODE == 1 || MODE == 2, HALF = MODE == 2;
     using L = RL<M>;
     using B = BX<M>;
     constexpr int Q = 2 * M + 1;
@@ -696,6 +693,13 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
             st2(fx, q, o[0][3], o[1][3]);
             st2(fy, q, o[0][4], o[1][4]);
             st2(fz, q, o[0][5], o[1][5]);
+            if constexpr (MODE == 3) {
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    st2(hh.f[c], q, gp[0][c], gp[1][c]);
+                    st2(hh.f[3 + c], q, gr[0][c], gr[1][c]);
+                }
+            }
             if constexpr (HALF) {
                 const float ih2 = ih * ih;
                 st2(hh.f[0], q, hp0.x * hr0.x * ih2, hp0.y * hr0.y * ih2);
@@ -717,7 +721,7 @@ __global__ void __launch_bounds__(NTP, occ(MODE == 2 && M > 6 ? 1 : 2))
 tti_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__restrict__ r,
             const __grid_constant__ RMaps mp, float *__restrict__ ex, float *__restrict__ ey,
             float *__restrict__ ez, float *__restrict__ fx, float *__restrict__ fy, float *__restrict__ fz,
-            F3 hh, const __grid_constant__ RecDev rec, int xc, int *err)
+            F6 hh, const __grid_constant__ RecDev rec, int xc, int *err)
 {
     if (MODE == 0 && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
     tti_rot_body<M, MODE>(g, w, p, r, mp, ex, ey, ez, fx, fy, fz, hh, blockIdx.x, blockIdx.y, blockIdx.z, xc,
@@ -962,7 +966,7 @@ tti_rot_batch(const TtiShot *__restrict__ shots, const int4 *__restrict__ tiles,
 {
     const int4 tl = tiles[blockIdx.x];
     const TtiShot &S = shots[tl.x];
-    tti_rot_body<M, 0>(S.g, w, S.rp, S.rr, S.rm, S.t[0], S.t[1], S.t[2], S.t[3], S.t[4], S.t[5], F3{}, tl.y, tl.z,
+    tti_rot_body<M, 0>(S.g, w, S.rp, S.rr, S.rm, S.t[0], S.t[1], S.t[2], S.t[3], S.t[4], S.t[5], F6{}, tl.y, tl.z,
                            tl.w, S.xc, S.flag);
 }
 
@@ -1291,7 +1295,7 @@ int tti_launch(prop_s *P, float *const *S, const float *up, const float *ur, flo
     (void)attr;
     const RecDev rec = ADJ ? RecDev{} : P->rec;
     const dim3 grd1(grd.x, grd.y, grd.z + receiver_layers(rec, grd, blk));
-    launch_pass(tti_rot_tma<M>, grd1, blk, s1, P->stream, g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
+    launch_pass(tti_rot_tma<M>, grd1, blk, s1, P->stream, g, P->w, rp_, rr_, rm, t[0], t[1], t[2], t[3], t[4], t[5], F6{},
                                                 rec, xc, P->flag);
     launch_pass(tti_upd_tma<M, ADJ, GRAD>, grd, blk, s2, P->stream, g, P->w, t[0], t[3], um, pn, rn, grad, t[6], t[7],
                                                           P->flag, P->d.check_nan, ADJ ? InjDev{} : P->inj, xc,
@@ -1359,8 +1363,8 @@ __global__ void tti_axis_finalize(long long n, const float *th, const float *ph,
 // field (up, ur) at level n and the adjoint field (lp, lr) at level n+1:
 // rotation pass on the forward field, then the update pass in mode 2.
 // gax != NULL: also the tilt/azimuth term, from zeta = C lam in tmp[6], tmp[7]
-// (raw rotation passes on zeta into tmp[0..5] and on the forward field into
-// tmp[8..13], then tti_axis_image into gax[0..2])
+// (the rotation pass on the forward field leaves its raw derivatives in tmp[8..13],
+// a raw pass on zeta those in tmp[0..5], then tti_axis_image into gax[0..2])
 template <int M>
 int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp, const float *lr, float *ge,
                     float *gd, float *const *gax)
@@ -1384,8 +1388,15 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
     const size_t s1 = ring_smem(P, grd, occ(2), RL<M>::SZ, RL<M>::NS), s2 = ring_smem(P, grd, occ(2), UL<M, 2, 0>::SZ, NSTAGE);
     static const bool attr = set_smem(tti_rot_tma<M>, SMEM_MAX) && set_smem(tti_upd_tma<M, 2, 0>, SMEM_MAX);
     (void)attr;
-    launch_pass(tti_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5], F3{},
-                                               RecDev{}, xc, P->flag);
+    if (gax) {
+        static const bool attr3 = set_smem(tti_rot_tma<M, 3>, SMEM_MAX);
+        (void)attr3;
+        launch_pass(tti_rot_tma<M, 3>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5],
+                    F6{{t[8], t[9], t[10], t[11], t[12], t[13]}}, RecDev{}, xc, P->flag);
+    } else {
+        launch_pass(tti_rot_tma<M>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[0], t[1], t[2], t[3], t[4], t[5],
+                    F6{}, RecDev{}, xc, P->flag);
+    }
     launch_pass(tti_upd_tma<M, 2, 0>, grd, blk, s2, P->stream, g, P->w, t[0], t[3], um, nullptr, nullptr, ge, gd, nullptr,
                                                      P->flag, 0, InjDev{}, xc, P->flag);
     P->kern_launches += 2;
@@ -1398,9 +1409,7 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
         static const bool attr_raw = set_smem(tti_rot_tma<M, 1>, SMEM_MAX);
         (void)attr_raw;
         launch_pass(tti_rot_tma<M, 1>, grd, blk, s1, P->stream, g, P->w, t[6], t[7], rz, t[0], t[1], t[2], t[3], t[4], t[5],
-                                                       F3{}, RecDev{}, xc, P->flag);
-        launch_pass(tti_rot_tma<M, 1>, grd, blk, s1, P->stream, g, P->w, up, ur, rm, t[8], t[9], t[10], t[11], t[12], t[13],
-                                                       F3{}, RecDev{}, xc, P->flag);
+                                                       F6{}, RecDev{}, xc, P->flag);
         AxisIn ai;
         for (int c = 0; c < 6; c++) {
             ai.dz[c] = t[c];
@@ -1411,7 +1420,7 @@ int tti_image_aniso(prop_s *P, const float *up, const float *ur, const float *lp
         for (int c = 0; c < 3; c++) ai.acc[c] = gax[c];
         const long long n = (long long)g.N;
         tti_axis_image<<<(unsigned)((n + 255) / 256), 256, 0, P->stream>>>(n, P->g.dt * P->g.dt, ai);
-        P->kern_launches += 3;
+        P->kern_launches += 2;
     }
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
@@ -1491,7 +1500,7 @@ int raw_half(prop_s *P, const float *p, const float *r, float *const *dp, float 
     static const bool attr = set_smem(tti_rot_tma<M, 2>, s1);
     (void)attr;
     launch_pass(tti_rot_tma<M, 2>, grd, blk, s1, P->stream, g, P->w, p, r, rm, dp[0], dp[1], dp[2], dr[0], dr[1], dr[2],
-                                                   F3{{h[0], h[1], h[2]}}, RecDev{}, xc, P->flag);
+                                                   F6{{h[0], h[1], h[2]}}, RecDev{}, xc, P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
