@@ -662,8 +662,10 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
             const float2 n0 = lds2(S + L::ON + ii), n1 = lds2(S + L::ON + IS + ii);
             const float ih = g.ih;
             const unsigned q = x * pl + q0;
-            const float gp[2][3] = {{gp0a * ih, gp1a * ih, gp2a * ih}, {gp0b * ih, gp1b * ih, gp2b * ih}};
-            const float gr[2][3] = {{gr0a * ih, gr1a * ih, gr2a * ih}, {gr0b * ih, gr1b * ih, gr2b * ih}};
+            const float gp[2][3] = {{__fmul_rn(gp0a, ih), __fmul_rn(gp1a, ih), __fmul_rn(gp2a, ih)},
+                                    {__fmul_rn(gp0b, ih), __fmul_rn(gp1b, ih), __fmul_rn(gp2b, ih)}};
+            const float gr[2][3] = {{__fmul_rn(gr0a, ih), __fmul_rn(gr1a, ih), __fmul_rn(gr2a, ih)},
+                                    {__fmul_rn(gr0b, ih), __fmul_rn(gr1b, ih), __fmul_rn(gr2b, ih)}};
             const float nx2[2] = {n0.x, n0.y}, ny2[2] = {n1.x, n1.y};
             float o[2][6];
 #pragma unroll
@@ -676,13 +678,15 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
                     }
                     continue;
                 }
+                // spelt out: which products are fused must not depend on the mode, the
+                // tile height or the build
                 const float a0 = nx2[i], a1 = ny2[i];
-                const float a2 = sqrtf(fmaxf(0.f, 1.f - a0 * a0 - a1 * a1));
-                const float wpn = a0 * gp[i][0] + a1 * gp[i][1] + a2 * gp[i][2];
-                const float wrn = a0 * gr[i][0] + a1 * gr[i][1] + a2 * gr[i][2];
-                o[i][0] = gp[i][0] - a0 * wpn;
-                o[i][1] = gp[i][1] - a1 * wpn;
-                o[i][2] = gp[i][2] - a2 * wpn;
+                const float a2 = sqrtf(fmaxf(0.f, __fmaf_rn(-a1, a1, __fmaf_rn(-a0, a0, 1.f))));
+                const float wpn = __fmaf_rn(a2, gp[i][2], __fmaf_rn(a0, gp[i][0], __fmul_rn(a1, gp[i][1])));
+                const float wrn = __fmaf_rn(a2, gr[i][2], __fmaf_rn(a0, gr[i][0], __fmul_rn(a1, gr[i][1])));
+                o[i][0] = __fmaf_rn(-a0, wpn, gp[i][0]);
+                o[i][1] = __fmaf_rn(-a1, wpn, gp[i][1]);
+                o[i][2] = __fmaf_rn(-a2, wpn, gp[i][2]);
                 o[i][3] = a0 * wrn;
                 o[i][4] = a1 * wrn;
                 o[i][5] = a2 * wrn;
