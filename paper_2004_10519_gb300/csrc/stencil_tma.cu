@@ -6,7 +6,8 @@
 // shared-memory taps and global accesses are 8-byte (float2) and every y-tap
 // row serves two outputs.  For every plane the y/z-halo boxes of the differentiated fields
 // are fetched with cp.async.bulk.tensor into a shared-memory ring of three
-// stages (four in the TTI rotation and acoustic forward passes); out-of-grid
+// stages (four in the TTI rotation and acoustic forward passes; up to eight
+// where the grid leaves an SM the memory, ring_smem in tma.cuh); out-of-grid
 // elements arrive as zeros, which is the zero extension of the
 // finite-difference operators.  Every other per-plane input (the thread's
 // own values, parameters, the new head of each x-derivative queue M planes
@@ -344,7 +345,7 @@ WP_DEV void t_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, 
 
 template <int M, int MODE>
 WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, const float *S, const ElCtx<M> &t,
-                    int x, float2 (&qvx)[2 * M], float2 (&qvy)[2 * M], float2 (&qvz)[2 * M])
+                    int x, const float2 (&ep)[3], float2 (&qvx)[2 * M], float2 (&qvy)[2 * M], float2 (&qvz)[2 * M])
 {
     using L = TL<M, MODE>;
     using B = BX<M>;
@@ -422,16 +423,17 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, co
                 const float a3 = gxy0 * (t3.x - c * gxya), b3 = t.two ? gxy1 * (t3.y - c * gxyb) : 0.f;
                 const float a4 = gxz0 * (t4.x - c * gxza), b4 = t.two ? gxz1 * (t4.y - c * gxzb) : 0.f;
                 const float a5 = gyz0 * (t5.x - c * gyza), b5 = t.two ? gyz1 * (t5.y - c * gyzb) : 0.f;
-                const float la = l.x * (a0 + a1 + a2), lb = l.y * (b0 + b1 + b2);
+                // spelt out: the single and batched passes and the checking build round alike
+                const float la = __fmul_rn(l.x, a0 + a1 + a2), lb = __fmul_rn(l.y, b0 + b1 + b2);
                 st2(s.f[3], q, a0, b0);
                 st2(s.f[4], q, a1, b1);
                 st2(s.f[5], q, a2, b2);
                 st2(s.f[6], q, a3, b3);
                 st2(s.f[7], q, a4, b4);
                 st2(s.f[8], q, a5, b5);
-                st2(o.f[0], q, la + m2a * a0, lb + m2b * b0);
-                st2(o.f[1], q, la + m2a * a1, lb + m2b * b1);
-                st2(o.f[2], q, la + m2a * a2, lb + m2b * b2);
+                st2(o.f[0], q, __fmaf_rn(m2a, a0, la), __fmaf_rn(m2b, b0, lb));
+                st2(o.f[1], q, __fmaf_rn(m2a, a1, la), __fmaf_rn(m2b, b1, lb));
+                st2(o.f[2], q, __fmaf_rn(m2a, a2, la), __fmaf_rn(m2b, b2, lb));
                 st2(o.f[3], q, mxya * a3, mxyb * b3);
                 st2(o.f[4], q, mxza * a4, mxzb * b4);
                 st2(o.f[5], q, myza * a5, myzb * b5);
@@ -443,12 +445,9 @@ WP_DEV void t_plane(const GridDev &g, const FDW &w, const F9 &s, const F6 &o, co
             st2(o.f[1], q, gm.x + 2.f * c * (t0.x * exa + t1.x * eya + t2.x * eza),
                 gm.y + 2.f * c * (t0.y * exb + t1.y * eyb + t2.y * ezb));
             // edge products summed over the steps (gathered onto the nodes at the end)
-            const float2 p3 = *reinterpret_cast<const float2 *>(o.f[2] + q);
-            const float2 p4 = *reinterpret_cast<const float2 *>(o.f[3] + q);
-            const float2 p5 = *reinterpret_cast<const float2 *>(o.f[4] + q);
-            st2(o.f[2], q, p3.x + c * t3.x * gxya, p3.y + c * t3.y * gxyb);
-            st2(o.f[3], q, p4.x + c * t4.x * gxza, p4.y + c * t4.y * gxzb);
-            st2(o.f[4], q, p5.x + c * t5.x * gyza, p5.y + c * t5.y * gyzb);
+            st2(o.f[2], q, ep[0].x + c * t3.x * gxya, ep[0].y + c * t3.y * gxyb);
+            st2(o.f[3], q, ep[1].x + c * t4.x * gxza, ep[1].y + c * t4.y * gxzb);
+            st2(o.f[4], q, ep[2].x + c * t5.x * gyza, ep[2].y + c * t5.y * gyzb);
         }
     }
 #pragma unroll
@@ -489,11 +488,19 @@ WP_DEV void el_tpass_body(const GridDev &g, const FDW &w, const F9 &s, const F6 
     float2 qvx[Q], qvy[Q], qvz[Q];
     t_preload<M>(g, s, t, xa, qvx, qvy, qvz);
     for (int x = xa; x < xb; x++) {
+        // imaging: the edge sums of the plane, asked for before the wait for its
+        // ring stage (elastic gradient, 200^3 so 8: 25.1 -> 24.6 ms with their
+        // latency hidden; in the ring they would leave one CTA to an SM)
+        float2 ep[3];
+        if (MODE == 2 && t.act) {
+            const unsigned q = x * (unsigned)g.NY * (unsigned)g.PZ + t.q0;
+            for (int i = 0; i < 3; i++) ep[i] = *reinterpret_cast<const float2 *>(o.f[2 + i] + q);
+        }
         if (!__all_sync(0xffffffffu, R.wait_full())) {
             if (lane == 0) atomicOr(err, 2);
             return;
         }
-        t_plane<M, MODE>(g, w, s, o, sm + R.st * L::SZ, t, x, qvx, qvy, qvz);
+        t_plane<M, MODE>(g, w, s, o, sm + R.st * L::SZ, t, x, ep, qvx, qvy, qvz);
         R.release(lane);
     }
     if (MODE == 0 && inj && t.act)
