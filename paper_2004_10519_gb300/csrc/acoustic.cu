@@ -4,8 +4,9 @@
 //   u^{n+1} = (dt^2 L u^n + 2 m u^n - B u^{n-1}) / A,  A, B = m (1 +- sig dt/2),
 // L = sum over axes of the centred second derivative of the space order.
 // L is symmetric, so the transposed step is the same map.  The TMA-fed pass
-// (stencil_tma.cu) runs when NZ % 4 == 0; this file holds the dispatch and
-// a direct-load kernel for any NZ.
+// (stencil_tma.cu) runs on rows of whole 16-byte units (row_pitch in
+// runtime.cu); this file holds the dispatch and a direct-load kernel for any
+// row pitch.
 #include "tile.cuh"
 
 namespace {

@@ -5,8 +5,8 @@
 //   stress pass    tau <- g (tau + dt C S(v))
 // The transposed step (adjoint modelling) is the same two passes with
 // dt -> -dt in the variables (b_avg vbar, g C tbar).  These kernels serve
-// grids whose computational NZ is not a multiple of 4 (the TMA-fed passes
-// need 16-byte rows).
+// handles that the TMA-fed passes do not (tma_usable: rows that row_pitch
+// leaves unpadded, 16-bit checkpoints on ragged rows, WAVEPROP_NO_TMA).
 //
 // Pipelining: while plane x is computed from shared memory, the loads of
 // plane x+1 (x-queue heads, own interior values, an even share of the halo

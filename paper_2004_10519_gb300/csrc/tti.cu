@@ -15,9 +15,9 @@
 // The adjoint step is the transpose: C is applied BEFORE the stencil
 // (L^T = H C); pass (1) forms zeta = C lam while loading.
 //
-// The passes themselves live in stencil_tma.cu (TMA-fed, NZ a multiple of
-// 4) and tti_fast.cu (pipelined loads, any NZ); this file dispatches a step
-// and sizes the x-chunks of the streaming kernels.
+// The passes themselves live in stencil_tma.cu (TMA-fed, a row pitch of a
+// multiple of 4) and tti_fast.cu (pipelined loads, any pitch); this file
+// dispatches a step and sizes the x-chunks of the streaming kernels.
 #include "common.cuh"
 
 #include <algorithm>
