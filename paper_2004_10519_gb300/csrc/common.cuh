@@ -40,9 +40,10 @@ WP_DEV float ldz(const float *__restrict__ f, const GridDev &g, int x, int y, in
     return (x >= 0 && x < g.NX && y >= 0 && y < g.NY && z >= 0 && z < g.NZ) ? __ldg(f + gidx(g, x, y, z)) : 0.f;
 }
 
-// one receiver: the weighted sum over its corners
-WP_DEV float record_point(const long long *__restrict__ idx, const float *__restrict__ w, int i,
-                          const float *__restrict__ f0, const float *__restrict__ f1, const float *__restrict__ f2)
+// one receiver: the weighted sum over its corners (the fields without restrict: a
+// pass that samples may have been launched while they were written)
+WP_DEV float record_point(const long long *__restrict__ idx, const float *__restrict__ w, int i, const float *f0,
+                          const float *f1, const float *f2)
 {
     float s = 0.f;
 #pragma unroll

@@ -142,9 +142,9 @@ WP_DEV void v_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, 
 #pragma unroll
     for (int j = 0; j < 2 * M - 1; j++) {
         const int xq = xa - M + 1 + j, xr = xa - M + j;
-        qxx[j] = t.act && xq >= 0 && xq < g.NX ? ldg2(s.f[3], xq * pl + t.q0) : Z2;
-        qxy[j] = t.act && xr >= 0 && xr < g.NX ? ldg2(s.f[6], xr * pl + t.q0) : Z2;
-        qxz[j] = t.act && xr >= 0 && xr < g.NX ? ldg2(s.f[7], xr * pl + t.q0) : Z2;
+        qxx[j] = t.act && xq >= 0 && xq < g.NX ? ldf2(s.f[3], xq * pl + t.q0) : Z2;
+        qxy[j] = t.act && xr >= 0 && xr < g.NX ? ldf2(s.f[6], xr * pl + t.q0) : Z2;
+        qxz[j] = t.act && xr >= 0 && xr < g.NX ? ldf2(s.f[7], xr * pl + t.q0) : Z2;
     }
 }
 
@@ -337,9 +337,9 @@ WP_DEV void t_preload(const GridDev &g, const F9 &s, const ElCtx<M> &t, int xa, 
 #pragma unroll
     for (int j = 0; j < 2 * M - 1; j++) {
         const int xr = xa - M + j, xq = xa - M + 1 + j;
-        qvx[j] = t.act && xr >= 0 && xr < g.NX ? ldg2(s.f[0], xr * pl + t.q0) : Z2;
-        qvy[j] = t.act && xq >= 0 && xq < g.NX ? ldg2(s.f[1], xq * pl + t.q0) : Z2;
-        qvz[j] = t.act && xq >= 0 && xq < g.NX ? ldg2(s.f[2], xq * pl + t.q0) : Z2;
+        qvx[j] = t.act && xr >= 0 && xr < g.NX ? ldf2(s.f[0], xr * pl + t.q0) : Z2;
+        qvy[j] = t.act && xq >= 0 && xq < g.NX ? ldf2(s.f[1], xq * pl + t.q0) : Z2;
+        qvz[j] = t.act && xq >= 0 && xq < g.NX ? ldf2(s.f[2], xq * pl + t.q0) : Z2;
     }
 }
 
@@ -574,11 +574,10 @@ struct RMaps {
 
 // one tile (bx, by: 32 z x FY y columns; bz: x chunk of xc planes)
 template <int M, int MODE>
-WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict__ p,
-                         const float *__restrict__ r, const RMaps &mp, float *__restrict__ ex,
-                         float *__restrict__ ey, float *__restrict__ ez, float *__restrict__ fx,
-                         float *__restrict__ fy, float *__restrict__ fz, const F6 &hh, int bx, int by, int bz,
-                         int xc, int *err)
+WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *p, const float *r, const RMaps &mp,
+                         float *__restrict__ ex, float *__restrict__ ey, float *__restrict__ ez,
+                         float *__restrict__ fx, float *__restrict__ fy, float *__restrict__ fz, const F6 &hh, int bx,
+                         int by, int bz, int xc, int *err)
 {
     constexpr bool RAW = MODE == 1 || MODE == 2, HALF = MODE == 2;
     using L = RL<M>;
@@ -624,8 +623,8 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
     for (int j = 0; j < Q - 1; j++) {
         const int xq = xa - M + j;
         const bool in = act && xq >= 0 && xq < g.NX;
-        qp[j] = in ? ldg2(p, xq * pl + q0) : Z2;
-        qr[j] = in ? ldg2(r, xq * pl + q0) : Z2;
+        qp[j] = in ? ldf2(p, xq * pl + q0) : Z2;
+        qr[j] = in ? ldf2(r, xq * pl + q0) : Z2;
     }
     const int cy = ty + M, cz = B::MZ + 2 * tz, ii = ty * FZ + 2 * tz;
     const int ci = cy * B::RC + cz;
@@ -729,10 +728,9 @@ WP_DEV void tti_rot_body(const GridDev &g, const FDW &w, const float *__restrict
 
 template <int M, int MODE = 0>
 __global__ void __launch_bounds__(NTP, occ(MODE == 2 && M > 6 ? 1 : 2))
-tti_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__restrict__ r,
-            const __grid_constant__ RMaps mp, float *__restrict__ ex, float *__restrict__ ey,
-            float *__restrict__ ez, float *__restrict__ fx, float *__restrict__ fy, float *__restrict__ fz,
-            F6 hh, const __grid_constant__ RecDev rec, int xc, int *err)
+tti_rot_tma(GridDev g, FDW w, const float *p, const float *r, const __grid_constant__ RMaps mp,
+            float *__restrict__ ex, float *__restrict__ ey, float *__restrict__ ez, float *__restrict__ fx,
+            float *__restrict__ fy, float *__restrict__ fz, F6 hh, const __grid_constant__ RecDev rec, int xc, int *err)
 {
     if (MODE == 0 && sample_receivers(rec, (g.NX + xc - 1) / xc)) return;
     tti_rot_body<M, MODE>(g, w, p, r, mp, ex, ey, ez, fx, fy, fz, hh, blockIdx.x, blockIdx.y, blockIdx.z, xc,
@@ -774,9 +772,8 @@ struct UMaps {
 };
 
 template <int M, int ADJ, int GRAD>
-WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict__ ex,
-                         const float *__restrict__ fx, const UMaps &mp, float *__restrict__ pp,
-                         float *__restrict__ rp, float *__restrict__ grad, float *__restrict__ zp,
+WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *ex, const float *fx, const UMaps &mp,
+                         float *pp, float *rp, float *__restrict__ grad, float *__restrict__ zp,
                          float *__restrict__ zr, int *flag, int check, const InjDev *inj, int bx, int by, int bz,
                          int xc, int *err)
 {
@@ -841,8 +838,8 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
     for (int j = 0; j < Q - 1; j++) {
         const int xq = xa - M + j;
         const bool in = act && xq >= 0 && xq < g.NX;
-        qe[j] = in ? ldg2(ex, xq * pl + q0) : Z2;
-        qf[j] = in ? ldg2(fx, xq * pl + q0) : Z2;
+        qe[j] = in ? ldf2(ex, xq * pl + q0) : Z2;
+        qf[j] = in ? ldf2(fx, xq * pl + q0) : Z2;
     }
     const float *sx = g.tab, *sy = g.tab + g.NX, *sz = g.tab + g.NX + g.NY;
     const float dt2 = g.dt * g.dt, hdt = 0.5f * g.dt;
@@ -943,9 +940,8 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *__restrict
 
 template <int M, int ADJ, int GRAD>
 __global__ void __launch_bounds__(NTP, occ(2))
-tti_upd_tma(GridDev g, FDW w, const float *__restrict__ ex, const float *__restrict__ fx,
-            const __grid_constant__ UMaps mp, float *__restrict__ pp, float *__restrict__ rp,
-            float *__restrict__ grad, float *__restrict__ zp, float *__restrict__ zr, int *flag, int check,
+tti_upd_tma(GridDev g, FDW w, const float *ex, const float *fx, const __grid_constant__ UMaps mp, float *pp,
+            float *rp, float *__restrict__ grad, float *__restrict__ zp, float *__restrict__ zr, int *flag, int check,
             const __grid_constant__ InjDev inj, int xc, int *err)
 {
     tti_upd_body<M, ADJ, GRAD>(g, w, ex, fx, mp, pp, rp, grad, zp, zr, flag, check, &inj, blockIdx.x, blockIdx.y,
@@ -1028,7 +1024,7 @@ struct AMaps {
 
 template <int M, int GRAD>
 __global__ void __launch_bounds__(NTP, M <= 6 ? 2 : 1)
-acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, float *__restrict__ grad,
+acu_tma(GridDev g, FDW w, const float *u1, float *u0, float *__restrict__ grad,
         const __grid_constant__ AMaps mp, int *flag, int check, const __grid_constant__ RecDev rec,
         const __grid_constant__ InjDev inj, int xc, int *err)
 {
@@ -1078,8 +1074,8 @@ acu_tma(GridDev g, FDW w, const float *__restrict__ u1, float *__restrict__ u0, 
     for (int j = 0; j < Q - 1; j++) {
         const int xq = xa - M + j;
         const bool in = xq >= 0 && xq < g.NX;
-        qu0[j] = a0 && in ? ldg2(u1, xq * pl + qa) : Z2;
-        qu1[j] = a1 && in ? ldg2(u1, xq * pl + qb) : Z2;
+        qu0[j] = a0 && in ? ldf2(u1, xq * pl + qa) : Z2;
+        qu1[j] = a1 && in ? ldf2(u1, xq * pl + qb) : Z2;
     }
     const float *sx = g.tab, *sy = g.tab + g.NX, *sz = g.tab + g.NX + g.NY;
     const float sz0 = a0 ? __ldg(sz + z) : 0.f, sz1 = a0 ? __ldg(sz + min(z + 1, g.NZ - 1)) : 0.f;

@@ -150,12 +150,16 @@ WP_DEV float2 lds2(const float *p)
 #endif
     return *reinterpret_cast<const float2 *>(p);
 }
-WP_DEV float2 ldg2(const float *__restrict__ p, unsigned o)
+// a pair of a field that the kernel before may still be writing when this one
+// starts (launch_pass): an ordinary load, after pass_waits.  Never __ldg, nor
+// through a restrict pointer: read-only loads may move above the wait, and read
+// lines fetched before it
+WP_DEV float2 ldf2(const float *p, unsigned o)
 {
 #ifdef WP_CHECK
     if (!ck_field(o)) return make_float2(0.f, 0.f);
 #endif
-    return __ldg(reinterpret_cast<const float2 *>(p + o));
+    return *reinterpret_cast<const float2 *>(p + o);
 }
 WP_DEV void st2(float *p, unsigned o, float a, float b)
 {
@@ -218,7 +222,10 @@ WP_DEV void zwin(const float *row, int cz, float (&w)[2 * M + 2])
 // wait here, before they touch anything in memory, until that kernel has
 // completed and its writes are visible.  Hides the launch latency and the
 // prologue behind the last CTAs of the pass before.  No effect in a kernel
-// that was launched without the attribute.
+// that was launched without the attribute.  The fields of such a pass (what any
+// pass writes) come by TMA or ordinary loads, and its field pointers carry no
+// restrict, for only those are ordered by the wait; __ldg is for the model, the
+// layer tables, the sparse-point tables and the wavelets, which no pass writes.
 WP_DEV void pass_begins() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 WP_DEV void pass_waits() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -44,7 +44,7 @@ struct F12 {
 
 template <int M>
 __global__ void __launch_bounds__(NTP, M <= 6 ? 2 : 1)
-tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__restrict__ r,
+tti_sp_rot_tma(GridDev g, FDW w, const float *p, const float *r,
                const __grid_constant__ SRMaps mp, F12 o, int xc, int *err)
 {
     using L = SRL<M>;
@@ -91,8 +91,8 @@ tti_sp_rot_tma(GridDev g, FDW w, const float *__restrict__ p, const float *__res
     for (int j = 0; j < Q - 1; j++) {
         const int xq = xa - M + j;
         const bool in = act && xq >= 0 && xq < g.NX;
-        qp[j] = in ? ldg2(p, xq * pl + q0) : Z2;
-        qr[j] = in ? ldg2(r, xq * pl + q0) : Z2;
+        qp[j] = in ? ldf2(p, xq * pl + q0) : Z2;
+        qr[j] = in ? ldf2(r, xq * pl + q0) : Z2;
     }
     const int cy = ty + M, cz = B::MZ + 2 * tz, c2 = 2 * tz, ii = ty * FZ + c2;
     const int ci = cy * B::RC + cz;
@@ -277,8 +277,8 @@ WP_DEV float2 yz_part(const float *yc, const float *ys, const float *zc, const f
 
 template <int M, int ADJ, int GRAD>
 __global__ void __launch_bounds__(NTP, 1)
-tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float *__restrict__ pp,
-               float *__restrict__ rp, float *__restrict__ grad, float *__restrict__ zp, float *__restrict__ zr,
+tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float *pp, float *rp,
+               float *__restrict__ grad, float *__restrict__ zp, float *__restrict__ zr,
                int *flag, int check, int xc, int *err)
 {
     using L = SUL<M, ADJ, GRAD>;
@@ -349,8 +349,8 @@ tti_sp_upd_tma(GridDev g, FDW w, F12 o, const __grid_constant__ SUMaps mp, float
     for (int j = 0; j < 2 * M; j++) {
         const int xh = xa - M + j, xs = xh - 1;
         const bool ih_ = act && xh >= 0 && xh < g.NX, is_ = act && xs >= 0 && xs < g.NX;
-        push_x<M>(a0, ih_ ? ldg2(o.f[0], xh * pl + q0) : Z2, is_ ? ldg2(o.f[6], xs * pl + q0) : Z2, w);
-        push_x<M>(az, ih_ ? ldg2(o.f[3], xh * pl + q0) : Z2, is_ ? ldg2(o.f[9], xs * pl + q0) : Z2, w);
+        push_x<M>(a0, ih_ ? ldf2(o.f[0], xh * pl + q0) : Z2, is_ ? ldf2(o.f[6], xs * pl + q0) : Z2, w);
+        push_x<M>(az, ih_ ? ldf2(o.f[3], xh * pl + q0) : Z2, is_ ? ldf2(o.f[9], xs * pl + q0) : Z2, w);
         shift_x<M>(a0);
         shift_x<M>(az);
     }
