@@ -53,6 +53,7 @@ struct SparseDev {
     int *cell_ptr = nullptr; // [ncell+1]
     int *ent_trace = nullptr;
     float *ent_w = nullptr;
+    cudaStream_t stream = nullptr;   // that uses the tables
     int few = 0;             // ncell where it is at most INJ_MAX, with the cells' places
     int few_x[INJ_MAX] = {};
     unsigned few_o[INJ_MAX] = {};
@@ -379,9 +380,9 @@ int wp_fail(prop_s *P, int code, const std::string &msg);
 // records the failure on the handle (P may be NULL)
 int wp_dev_alloc(void **p, size_t bytes, const char *what, std::string *msg);
 int wp_malloc(prop_s *P, void **p, size_t bytes, const char *what);
-// frees what wp_dev_alloc gave (NULL-safe; synchronises the device); bytes that
-// the pool of device memory holds unused
-void wp_dev_free(void *p);
+// frees what wp_dev_alloc gave (NULL-safe) after synchronising the stream that
+// last used it; bytes that the pool of device memory holds unused
+void wp_dev_free(void *p, cudaStream_t used);
 size_t wp_dev_idle();
 // status of the device error word read back after a call: bit 3 (the
 // bounds-checking build skipped an access) -> PROP_ECUDA; bit 1 (a bounded

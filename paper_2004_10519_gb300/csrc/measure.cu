@@ -55,7 +55,7 @@ extern "C" int prop_fp32_peak(double *tflops)
     const cudaError_t err = cudaGetLastError();
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    wp_dev_free(out);
+    wp_dev_free(out, nullptr);
     if (err != cudaSuccess) return PROP_ECUDA;
     *tflops = best;
     return PROP_OK;

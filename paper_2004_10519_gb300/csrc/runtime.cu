@@ -53,8 +53,10 @@ int wp_cuda(prop_s *P, cudaError_t e, const char *what)
 // outside the library: the driver then takes unused pool memory back, checked
 // with a cudaMalloc of more than was free).  Its allocations and frees are
 // ordered on a stream of its own, where each allocation is waited for and each
-// free follows a device synchronisation (as cudaFree's), so memory passes
-// between streams and threads as with cudaMalloc.
+// free comes after a synchronisation of the stream that used the block, so memory
+// passes between streams and threads as with cudaMalloc.  Not of the device: that
+// is refused while any of its streams is being captured (prop_step and the
+// batches capture; so may the caller's other threads).
 namespace {
 struct DevPool {
     cudaMemPool_t pool = nullptr;
@@ -97,18 +99,28 @@ DevPool *dev_pool(int dev = -1)
 }
 }  // namespace
 
-void wp_dev_free(void *p)
+// free p, whose last use is on stream `used` of p's device; the current device may
+// be another one
+void wp_dev_free(void *p, cudaStream_t used)
 {
     if (!p) return;
     cudaPointerAttributes a;
-    DevPool *d = cudaPointerGetAttributes(&a, p) == cudaSuccess ? dev_pool(a.device) : nullptr;
-    if (!d) {
+    int cur = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&cur) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(p);
         return;
     }
-    cudaDeviceSynchronize();
-    cudaFreeAsync(p, d->st);
+    if (cur != a.device) cudaSetDevice(a.device);      // the default stream is the current device's
+    DevPool *d = dev_pool(a.device);
+    const cudaError_t e = cudaStreamSynchronize(used);
+    bool ok = e == cudaSuccess;
+    // a stream that the caller is capturing: what uses the block cannot be waited
+    // for, so it is not given to anyone else
+    const bool captured = e >= cudaErrorStreamCaptureUnsupported && e <= cudaErrorStreamCaptureWrongThread;
+    if (!captured && (!d || cudaFreeAsync(p, d->st) != cudaSuccess))
+        ok = cudaFree(p) == cudaSuccess && !d && ok;   // allocated without the pool
+    if (!ok) cudaGetLastError();
+    if (cur != a.device) cudaSetDevice(cur);
 }
 
 // bytes that the pool holds unused (free to the library's next allocations)
@@ -320,9 +332,17 @@ static bool is_dev(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-struct DevBuf {   // RAII device buffer owned by one call
+struct DevBuf {   // RAII device buffer owned by one call, used on the call's stream
     void *p = nullptr;
-    ~DevBuf() { wp_dev_free(p); }
+    cudaStream_t st = nullptr;
+    int alloc(prop_s *P, size_t bytes, const char *what)
+    {
+        st = P->stream;
+        return wp_malloc(P, &p, bytes, what);
+    }
+    DevBuf() = default;
+    DevBuf(const DevBuf &) = delete;
+    ~DevBuf() { wp_dev_free(p, st); }
 };
 
 // device view of a caller buffer of n floats (copied in if host)
@@ -332,7 +352,7 @@ static int dev_in(prop_s *P, const float *src, size_t n, DevBuf &tmp, const floa
         *out = src;
         return PROP_OK;
     }
-    WP_TRY(wp_malloc(P, &tmp.p, n * sizeof(float), "input staging"));
+    WP_TRY(tmp.alloc(P, n * sizeof(float), "input staging"));
     WP_CK(P, cudaMemcpyAsync(tmp.p, src, n * sizeof(float), cudaMemcpyHostToDevice, P->stream));
     *out = (const float *)tmp.p;
     return PROP_OK;
@@ -428,11 +448,11 @@ static int ensure_ast(prop_s *P)
 
 static void free_snaps(prop_s *P)
 {
-    wp_dev_free(P->tail); P->tail = nullptr; P->tail_bytes = 0; P->tail_T = 0;
-    wp_dev_free(P->snap); P->snap = nullptr; P->snap_bytes = 0;
-    wp_dev_free(P->snap16); P->snap16 = nullptr; P->snap16_bytes = 0;
-    wp_dev_free(P->snap_scale); P->snap_scale = nullptr;
-    wp_dev_free(P->seg); P->seg = nullptr; P->seg_bytes = 0;
+    wp_dev_free(P->tail, P->stream); P->tail = nullptr; P->tail_bytes = 0; P->tail_T = 0;
+    wp_dev_free(P->snap, P->stream); P->snap = nullptr; P->snap_bytes = 0;
+    wp_dev_free(P->snap16, P->stream); P->snap16 = nullptr; P->snap16_bytes = 0;
+    wp_dev_free(P->snap_scale, P->stream); P->snap_scale = nullptr;
+    wp_dev_free(P->seg, P->stream); P->seg = nullptr; P->seg_bytes = 0;
     P->saved = false;
     P->tmaps.clear();        // descriptors may name the freed buffers
 }
@@ -440,13 +460,13 @@ static void free_snaps(prop_s *P)
 static void free_all(prop_s *P)
 {
     float *arrs[] = {P->m, P->c1, P->c2, P->th, P->ph, P->nrm[0], P->nrm[1], P->bu, P->lam, P->mu, P->acw};
-    for (float *a : arrs) wp_dev_free(a);
-    for (auto &a : P->st) wp_dev_free(a);
-    for (auto &a : P->ast) wp_dev_free(a);
-    for (auto &a : P->tmp) wp_dev_free(a);
-    wp_dev_free(P->flag);
-    wp_dev_free(P->sumsq);
-    wp_dev_free(P->tab);
+    for (float *a : arrs) wp_dev_free(a, P->stream);
+    for (auto &a : P->st) wp_dev_free(a, P->stream);
+    for (auto &a : P->ast) wp_dev_free(a, P->stream);
+    for (auto &a : P->tmp) wp_dev_free(a, P->stream);
+    wp_dev_free(P->flag, P->stream);
+    wp_dev_free(P->sumsq, P->stream);
+    wp_dev_free(P->tab, P->stream);
     free_snaps(P);
     for (auto e : P->prof_ev) cudaEventDestroy(e);
     if (P->step_graph) cudaGraphExecDestroy(P->step_graph);
@@ -721,7 +741,8 @@ static int create_impl(prop_s *P, const prop_desc *d, const float *const *model)
     const size_t N = (size_t)g.N;
     float *phys = nullptr;
     WP_MALLOC(P, phys, np * sizeof(float), "model staging");
-    std::unique_ptr<void, decltype(&wp_dev_free)> guard(phys, &wp_dev_free);
+    auto free_phys = [P](void *p) { wp_dev_free(p, P->stream); };
+    std::unique_ptr<void, decltype(free_phys)> guard(phys, free_phys);
     auto upload = [&](int i, float *&dst, float scale, int mode) -> int {
         WP_MALLOC(P, dst, N * sizeof(float), "model");
         WP_CK(P, cudaMemcpyAsync(phys, hm[i].data(), np * sizeof(float), cudaMemcpyHostToDevice, P->stream));
@@ -1376,8 +1397,8 @@ static int forward_impl(prop_s *P, const float *wavelet, const float *src, int n
     DevBuf wbuf, stage, tr;
     const float *wav = nullptr;
     WP_TRY(dev_in(P, wavelet, (size_t)nsrc * nt, wbuf, &wav));
-    WP_TRY(wp_malloc(P, &stage.p, sizeof(float) * (size_t)nt * nrec, "trace staging"));
-    WP_TRY(wp_malloc(P, &tr.p, sizeof(float) * (size_t)nt * nrec, "traces"));
+    WP_TRY(stage.alloc(P, sizeof(float) * (size_t)nt * nrec, "trace staging"));
+    WP_TRY(tr.alloc(P, sizeof(float) * (size_t)nt * nrec, "traces"));
     if (save) {
         WP_TRY(alloc_saves(P));
         if (P->d.kind == PROP_ELASTIC) WP_TRY(ensure_tmp(P, 15));
@@ -1655,8 +1676,8 @@ extern "C" int prop_adjoint(prop_t *P, const float *traces_in, const float *rec_
     DevBuf rbuf, stage, out;
     const float *res = nullptr;
     WP_TRY(dev_in(P, traces_in, (size_t)nrec * nt, rbuf, &res));
-    WP_TRY(wp_malloc(P, &stage.p, sizeof(float) * (size_t)nt * nsrc, "source staging"));
-    WP_TRY(wp_malloc(P, &out.p, sizeof(float) * (size_t)nt * nsrc, "source output"));
+    WP_TRY(stage.alloc(P, sizeof(float) * (size_t)nt * nsrc, "source staging"));
+    WP_TRY(out.alloc(P, sizeof(float) * (size_t)nt * nsrc, "source output"));
     if (P->d.kind == PROP_TTI) WP_TRY(tti_sweep(P, G, res, nullptr, (float *)stage.p, nullptr));
     else if (P->d.kind == PROP_ACOUSTIC) WP_TRY(ac_sweep(P, G, res, nullptr, (float *)stage.p, nullptr));
     else if (P->d.kind == PROP_ELASTIC2D) WP_TRY(el2_sweep(P, G, res, (float *)stage.p));
@@ -1679,12 +1700,12 @@ static int backward_impl(prop_s *P, const float *resid, float *grad, float *src_
     DevBuf rbuf, wbuf, stage, out, gbuf, gphys;
     const float *res = nullptr;
     WP_TRY(dev_in(P, resid, (size_t)nrec * nt, rbuf, &res));
-    WP_TRY(wp_malloc(P, &wbuf.p, sizeof(float) * (size_t)nsrc * nt, "wavelet"));
+    WP_TRY(wbuf.alloc(P, sizeof(float) * (size_t)nsrc * nt, "wavelet"));
     WP_CK(P, cudaMemcpyAsync(wbuf.p, P->saved_wav.data(), sizeof(float) * (size_t)nsrc * nt,
                              cudaMemcpyHostToDevice, P->stream));
     if (src_grad) {
-        WP_TRY(wp_malloc(P, &stage.p, sizeof(float) * (size_t)nt * nsrc, "source staging"));
-        WP_TRY(wp_malloc(P, &out.p, sizeof(float) * (size_t)nt * nsrc, "source output"));
+        WP_TRY(stage.alloc(P, sizeof(float) * (size_t)nt * nsrc, "source staging"));
+        WP_TRY(out.alloc(P, sizeof(float) * (size_t)nt * nsrc, "source output"));
     }
     // computational-grid accumulators and physical outputs: TTI m (+ eps,
     // delta and the three dJ/dn components that become theta, phi); elastic
@@ -1695,10 +1716,10 @@ static int backward_impl(prop_s *P, const float *resid, float *grad, float *src_
     const size_t N = (size_t)P->g.N, np = (size_t)P->g.px * P->g.py * P->g.pz;
     float *g3[6] = {};
     if (grad) {
-        WP_TRY(wp_malloc(P, &gbuf.p, sizeof(float) * N * ng, "gradient"));
+        WP_TRY(gbuf.alloc(P, sizeof(float) * N * ng, "gradient"));
         WP_CK(P, cudaMemsetAsync(gbuf.p, 0, sizeof(float) * N * ng, P->stream));
         for (int i = 0; i < ng; i++) g3[i] = (float *)gbuf.p + i * N;
-        WP_TRY(wp_malloc(P, &gphys.p, sizeof(float) * np * nout, "gradient (physical)"));
+        WP_TRY(gphys.alloc(P, sizeof(float) * np * nout, "gradient (physical)"));
     }
     if (P->d.kind == PROP_TTI)
         WP_TRY(tti_sweep(P, G, res, (const float *)wbuf.p, (float *)stage.p, grad ? g3 : nullptr));
@@ -1781,9 +1802,9 @@ static int trim_work(prop_s *P)
     WP_TRY(check_usable(P));      // launches nothing: the launch count stays
     WP_CK(P, cudaStreamSynchronize(P->stream));
     free_snaps(P);
-    for (auto &a : P->st) { wp_dev_free(a); a = nullptr; }
-    for (auto &a : P->ast) { wp_dev_free(a); a = nullptr; }
-    for (auto &a : P->tmp) { wp_dev_free(a); a = nullptr; }
+    for (auto &a : P->st) { wp_dev_free(a, P->stream); a = nullptr; }
+    for (auto &a : P->ast) { wp_dev_free(a, P->stream); a = nullptr; }
+    for (auto &a : P->tmp) { wp_dev_free(a, P->stream); a = nullptr; }
     P->saved = false;
     P->tmaps.clear();
     if (P->step_graph) {
@@ -1861,7 +1882,7 @@ extern "C" int prop_gradient(prop_t *P, const float *wavelet, const float *src_x
     if (!d_obs || !grad) return wp_fail(P, PROP_EINVAL, "d_obs or grad is NULL");
     const int nt = P->d.nt;
     DevBuf tr, obs;
-    WP_TRY(wp_malloc(P, &tr.p, sizeof(float) * (size_t)nrec * nt, "traces"));
+    WP_TRY(tr.alloc(P, sizeof(float) * (size_t)nrec * nt, "traces"));
     int rc = forward_impl(P, wavelet, src_xyz, nsrc, rec_xyz, nrec, (float *)tr.p, true);
     if (rc) { free_snaps(P); return rc; }
     const float *dobs = nullptr;
@@ -2161,12 +2182,12 @@ extern "C" int prop_forward_batch(prop_t *const *shots, int n, const float *cons
         prop_s *P = shots[i];
         WP_TRY(build_geometry(P, G[i], src_xyz[i], nsrc[i], rec_xyz[i], nrec[i]));
         WP_TRY(dev_in(P, wavelet[i], (size_t)nsrc[i] * nt, wb[i], &wav[i]));
-        WP_TRY(wp_malloc(P, &stage[i].p, sizeof(float) * (size_t)nt * nrec[i], "trace staging"));
-        WP_TRY(wp_malloc(P, &tr[i].p, sizeof(float) * (size_t)nt * nrec[i], "traces"));
+        WP_TRY(stage[i].alloc(P, sizeof(float) * (size_t)nt * nrec[i], "trace staging"));
+        WP_TRY(tr[i].alloc(P, sizeof(float) * (size_t)nt * nrec[i], "traces"));
         WP_TRY(zero_fields(P, P->st, nfields(P)));
     }
     DevBuf tbuf;
-    WP_TRY(wp_malloc(P0, &tbuf.p, sizeof(int), "time index"));
+    WP_TRY(tbuf.alloc(P0, sizeof(int), "time index"));
     int *tdev = (int *)tbuf.p;
     WP_CK(P0, cudaMemsetAsync(tdev, 0, sizeof(int), st));
     // TTI: the two buffer arrangements of a step, (p, r, p_prev, r_prev) and
@@ -2422,10 +2443,10 @@ static int gradient_lockstep(prop_t *const *shots, int n, const float *const *wa
         WP_TRY(build_geometry(P, G[i], src_xyz[i], nsrc[i], rec_xyz[i], nrec[i]));
         WP_TRY(dev_in(P, wavelet[i], (size_t)nsrc[i] * nt, wb[i], &wav[i]));
         WP_TRY(dev_in(P, d_obs[i], (size_t)nrec[i] * nt, ob[i], &obs[i]));
-        WP_TRY(wp_malloc(P, &stage[i].p, sizeof(float) * (size_t)nt * nrec[i], "trace staging"));
-        WP_TRY(wp_malloc(P, &tr[i].p, sizeof(float) * (size_t)nt * nrec[i], "traces"));
-        WP_TRY(wp_malloc(P, &gb[i].p, sizeof(float) * N, "gradient"));
-        WP_TRY(wp_malloc(P, &gp[i].p, sizeof(float) * np, "gradient (physical)"));
+        WP_TRY(stage[i].alloc(P, sizeof(float) * (size_t)nt * nrec[i], "trace staging"));
+        WP_TRY(tr[i].alloc(P, sizeof(float) * (size_t)nt * nrec[i], "traces"));
+        WP_TRY(gb[i].alloc(P, sizeof(float) * N, "gradient"));
+        WP_TRY(gp[i].alloc(P, sizeof(float) * np, "gradient (physical)"));
         WP_CK(P, cudaMemsetAsync(gb[i].p, 0, sizeof(float) * N, st));
         WP_TRY(alloc_saves(P));
         WP_TRY(zero_fields(P, P->st, 4));
@@ -2444,7 +2465,7 @@ static int gradient_lockstep(prop_t *const *shots, int n, const float *const *wa
     for (int i = 1; i < n; i++)
         if (ckpt_K(shots[i]) != K || ckpt_J(shots[i]) != J || ckpt_span(shots[i]) != span) return 1;
     DevBuf tbuf;
-    WP_TRY(wp_malloc(P0, &tbuf.p, sizeof(int), "time index"));
+    WP_TRY(tbuf.alloc(P0, sizeof(int), "time index"));
     int *tdev = (int *)tbuf.p;
     // fixed tables: slots 0, 1 the forward arrangements of the state (the
     // recomputation starts from the same arrangement in every segment);
@@ -2746,10 +2767,10 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
         WP_TRY(build_geometry(P, G[i], src_xyz[i], nsrc[i], rec_xyz[i], nrec[i]));
         WP_TRY(dev_in(P, wavelet[i], (size_t)nsrc[i] * nt, wb[i], &wav[i]));
         WP_TRY(dev_in(P, d_obs[i], (size_t)nrec[i] * nt, ob[i], &obs[i]));
-        WP_TRY(wp_malloc(P, &stage[i].p, sizeof(float) * (size_t)nt * nrec[i], "trace staging"));
-        WP_TRY(wp_malloc(P, &tr[i].p, sizeof(float) * (size_t)nt * nrec[i], "traces"));
-        WP_TRY(wp_malloc(P, &gb[i].p, sizeof(float) * N * 3, "gradient"));
-        WP_TRY(wp_malloc(P, &gp[i].p, sizeof(float) * np * 3, "gradient (physical)"));
+        WP_TRY(stage[i].alloc(P, sizeof(float) * (size_t)nt * nrec[i], "trace staging"));
+        WP_TRY(tr[i].alloc(P, sizeof(float) * (size_t)nt * nrec[i], "traces"));
+        WP_TRY(gb[i].alloc(P, sizeof(float) * N * 3, "gradient"));
+        WP_TRY(gp[i].alloc(P, sizeof(float) * np * 3, "gradient (physical)"));
         WP_CK(P, cudaMemsetAsync(gb[i].p, 0, sizeof(float) * N * 3, st));
         WP_TRY(alloc_saves(P));
         WP_TRY(zero_fields(P, P->st, 9));
@@ -2769,7 +2790,7 @@ static int el_gradient_lockstep(prop_t *const *shots, int n, const float *const 
         if (ckpt_K(shots[i]) != K || ckpt_J(shots[i]) != J || ckpt_span(shots[i]) != span) return 1;
     const int sf = (int)snap_fields(P0);
     DevBuf tbuf;
-    WP_TRY(wp_malloc(P0, &tbuf.p, sizeof(int), "time index"));
+    WP_TRY(tbuf.alloc(P0, sizeof(int), "time index"));
     int *tdev = (int *)tbuf.p;
     auto g3 = [&](int i, int c) { return (float *)gb[i].p + (size_t)c * shots[i]->g.N; };
     auto xs = [&](int i, int slot, const float **out) {

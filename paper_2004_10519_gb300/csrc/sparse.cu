@@ -411,6 +411,7 @@ int sp_build(prop_s *P, const float *xyz, int n, const int *trace_of_point, Spar
                  b_w = std::max<size_t>(1, T.ws.size()) * sizeof(float);
     const size_t total = up(b_ri) + up(b_rw) + up(b_c) + up(b_p) + up(b_t) + up(b_w);
     sp_free(S);
+    S->stream = P->stream;
     WP_TRY(wp_malloc(P, &S->blk, total, "sparse-point tables"));
     unsigned char *q = (unsigned char *)S->blk;
     S->rec_idx = (long long *)q; q += up(b_ri);
@@ -445,7 +446,7 @@ int sp_build(prop_s *P, const float *xyz, int n, const int *trace_of_point, Spar
 
 void sp_free(SparseDev *S)
 {
-    if (S->blk) wp_dev_free(S->blk);
+    wp_dev_free(S->blk, S->stream);
     *S = SparseDev{};
 }
 

@@ -1793,6 +1793,7 @@ struct TtiBatch {
     std::vector<int> elfixed_mode;
     size_t elfixed_cap = 0;
     FDW w{};
+    cudaStream_t st = nullptr;   // that the launches use
 };
 
 TtiBatch *tti_batch_new() { return new TtiBatch(); }
@@ -1800,11 +1801,11 @@ TtiBatch *tti_batch_new() { return new TtiBatch(); }
 void tti_batch_free(TtiBatch *b)
 {
     if (!b) return;
-    wp_dev_free(b->dtiles);
-    wp_dev_free(b->dshots);
-    for (auto d : b->dfixed) wp_dev_free(d);
-    for (auto d : b->elfixed) wp_dev_free(d);
-    wp_dev_free(b->del);
+    wp_dev_free(b->dtiles, b->st);
+    wp_dev_free(b->dshots, b->st);
+    for (auto d : b->dfixed) wp_dev_free(d, b->st);
+    for (auto d : b->elfixed) wp_dev_free(d, b->st);
+    wp_dev_free(b->del, b->st);
     for (int i = 0; i < TtiBatch::NSLOT; i++) {
         if (b->elcopied[i]) {
             cudaEventSynchronize(b->elcopied[i]);
@@ -1912,6 +1913,7 @@ static int tti_batch_tiles(TtiBatch *b, const TtiBatchReq *req, int n, cudaStrea
 }
 static int batch_tiles(TtiBatch *b, const std::vector<prop_s *> &Ps, cudaStream_t st, std::string *err)
 {
+    b->st = st;
     const int n = (int)Ps.size();
     auto ck = [&](cudaError_t c, const char *what) {
         if (c == cudaSuccess) return PROP_OK;
@@ -1938,7 +1940,7 @@ static int batch_tiles(TtiBatch *b, const std::vector<prop_s *> &Ps, cudaStream_
                 for (int z = 0; z < tz; z++) b->htiles.push_back(make_int4(i, z, y, c));
     }
     if (b->htiles.size() > b->tiles_cap) {
-        wp_dev_free(b->dtiles);
+        wp_dev_free(b->dtiles, st);
         b->dtiles = nullptr;
         b->tiles_cap = 0;
         if (int rc = wp_dev_alloc((void **)&b->dtiles, b->htiles.size() * sizeof(int4), "batched TTI tile table",
@@ -1973,7 +1975,7 @@ int tti_batch_fix(TtiBatch *b, const TtiBatchReq *req, int n, int slot, cudaStre
     if (int rc = tti_batch_tiles(b, req, n, st, err)) return rc;
     if ((size_t)n > b->fixed_cap) {              // every slot holds n entries
         for (auto &d : b->dfixed) {
-            wp_dev_free(d);
+            wp_dev_free(d, st);
             d = nullptr;
         }
         b->fixed_cap = n;
@@ -2065,7 +2067,7 @@ int tti_batch_step(TtiBatch *b, const TtiBatchReq *req, int n, cudaStream_t st, 
     };
     if (int rc = tti_batch_tiles(b, req, n, st, err)) return rc;
     if ((size_t)n > b->shots_cap) {
-        wp_dev_free(b->dshots);
+        wp_dev_free(b->dshots, st);
         b->dshots = nullptr;
         b->shots_cap = 0;
         if (int rc = wp_dev_alloc((void **)&b->dshots, n * sizeof(TtiShot), "batched TTI shot table", err)) return rc;
@@ -2171,7 +2173,7 @@ static int el_batch_launch(TtiBatch *b, const ElBatchReq *req, int n, cudaStream
     const int mode = req[0].mode, per = mode == 0 ? 1 : 3;
     const size_t bytes = (size_t)n * per * sizeof(ElShot);
     if (bytes > b->del_cap) {
-        wp_dev_free(b->del);
+        wp_dev_free(b->del, st);
         b->del = nullptr;
         b->del_cap = 0;
         if (int rc = wp_dev_alloc((void **)&b->del, bytes, "batched elastic shot table", err)) return rc;
@@ -2267,7 +2269,7 @@ int el_batch_fix(TtiBatch *b, const ElBatchReq *req, int n, int slot, cudaStream
     if (int rc = batch_tiles(b, Ps, st, err)) return rc;
     if ((size_t)n > b->elfixed_cap) {             // every slot holds 3n entries
         for (auto &d : b->elfixed) {
-            wp_dev_free(d);
+            wp_dev_free(d, st);
             d = nullptr;
         }
         b->elfixed_cap = n;

@@ -1,0 +1,67 @@
+"""The library's pool of device memory: blocks are freed after the work of the
+stream that used them, whatever other threads do meanwhile."""
+import glob
+import os
+import threading
+
+import numpy as np
+import pytest
+
+from test_gpu_rows import problem
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2004_10519_gb300", "csrc")
+
+
+def test_no_device_wide_synchronisation():
+    """It is refused while any stream of the device is captured, by another thread too: what it was to wait for
+    would not have been waited for."""
+    for f in glob.glob(os.path.join(CSRC, "*")):
+        with open(f) as src:
+            assert "cudaDeviceSynchronize" not in src.read(), f
+
+
+@pytest.mark.gpu
+def test_frees_beside_captures_of_another_thread(monkeypatch):
+    import paper_2004_10519_gb300 as wp
+    monkeypatch.setenv("WAVEPROP_GRAPHS", "1")           # prop_step must capture
+    p, q = problem("tti", 41), problem("elastic", 40, shape=(40, 33))
+    state = [np.random.default_rng(5).standard_normal((37, 43, 49), np.float32) for _ in range(4)]
+
+    def steps(prop):
+        out = []
+        for n in (4, 5, 7):
+            prop.set_state(state)
+            prop.step(n)
+            out += prop.get_state()
+            prop.trim()                                   # other buffers next time, so another capture
+        return out
+
+    def gradients(prop):
+        out = []
+        for scale in (0.5, 0.25, 0.0):
+            out.append(prop.gradient(q.wavelet, q.src, q.rec, scale * d)[0])
+            prop.trim()
+        return out
+
+    a, b = wp.Propagator.from_problem(p), wp.Propagator.from_problem(q, snap_mode=wp.SNAP_CKPT_FP32)
+    assert a.grid == state[0].shape
+    d = b.forward(q.wavelet, q.src, q.rec)
+    serial = steps(a), gradients(b)
+    got, errors = {}, []
+
+    def run(name, f, prop):
+        try:
+            got[name] = [f(prop) for _ in range(8)]
+        except Exception as e:                            # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=x) for x in (("steps", steps, a), ("gradients", gradients, b))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for name, ref in zip(("steps", "gradients"), serial):
+        for round_ in got[name]:
+            for x, y in zip(round_, ref):
+                np.testing.assert_array_equal(x, y)
