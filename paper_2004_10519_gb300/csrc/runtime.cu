@@ -634,10 +634,11 @@ extern "C" int prop_tile_rows(const prop_t *P) { return P ? P->tile_y : 0; }
 // run there too instead of on the pipelined passes.  Left as they are: rows so
 // short that the padding would be more than an eighth of them, grids that the
 // padding would take to 2^32 elements, and where a last bit of a wavefield
-// shows and the two families differ in it (the centred TTI passes do not): the
-// staggered-pair operators, whose FP32 error grows with the steps, and elastic
-// and acoustic handles with 16-bit checkpoints, whose rounding turns such a bit
-// into one of its own size.
+// shows and the two families differ in it (on padded rows the centred TTI and the
+// acoustic passes do not): the staggered-pair operators, whose FP32 error grows
+// with the steps, and elastic handles with 16-bit checkpoints, whose rounding turns
+// such a bit into one of its own size.  Acoustic handles with 16-bit checkpoints
+// are left there too.
 // Before and after, so 12, 281 x 267 x 193: TTI step 583 -> 350 us; so 8, 201 x
 // 171 x 139: elastic adjoint step 310 -> 136 us.
 void row_pitch(prop_s *P)

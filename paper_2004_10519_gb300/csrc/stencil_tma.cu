@@ -1001,8 +1001,8 @@ tti_upd_batch(const TtiShot *__restrict__ shots, const int4 *__restrict__ tiles,
 // paired FP32 arithmetic (__ffma2_rn and friends: per component the results
 // of the scalar operations).  The x loop is unrolled over the queue length,
 // so the x-derivative queues rotate by renaming instead of register moves.
-// stage: [u^n rect (y, z halo)] [queue head u^n (x+M)] [w, u^{n-1} (plane x)]
-//        (+ [u_f, g])
+// stage: [u^n rect (y, z halo)] [queue head u^n (x+M)] [w, or m where PAD,
+//        u^{n-1} (plane x)] (+ [u_f, g])
 // ---------------------------------------------------------------------------
 constexpr int AFY = 2 * FY;       // rows per CTA
 constexpr int AIS = FZ * AFY;     // interior box (floats)
@@ -1022,7 +1022,19 @@ struct AMaps {
     CUtensorMap u, q, w, u0, uf, g;
 };
 
-template <int M, int GRAD>
+// PAD: padded rows, whose handles ran acu_direct (acoustic.cu) before rows were
+// padded: its operations, A u^{n+1} = dt^2 L u^n + 2 m u^n - B u^{n-1} with the
+// model m in the place of w, in its order and with rounded quotients.  With the
+// form above they were less exact than before: a quotient by 1 + sd that is off by
+// a last bit is so at the same point in every step, which adds up in the layer (so
+// 4, 58 x 107 x 98 + 40, 130 steps: error of the state against 64 bits 2.2e-6 with
+// acu_direct and here, 3.4e-6 with the form above).  At 400 x 400 x 381, so 12 / 8 / 4:
+// acu_direct 1214 / 889 / 573 us a step, here 269 / 208 / 183, the form above 199 /
+// 173 / 165: the reciprocals and remainders are a third of the instructions at so
+// 12, which has 16 bytes of spills.  The reciprocals read from a field of their own
+// instead: 270 / 203 / 195 us, and 785 instead of 673 us for the two steps of a
+// gradient.
+template <int M, int GRAD, int PAD>
 __global__ void __launch_bounds__(NTP, M <= 6 ? 2 : 1)
 acu_tma(GridDev g, FDW w, const float *u1, float *u0, float *__restrict__ grad,
         const __grid_constant__ AMaps mp, int *flag, int check, const __grid_constant__ RecDev rec,
@@ -1080,7 +1092,10 @@ acu_tma(GridDev g, FDW w, const float *u1, float *u0, float *__restrict__ grad,
     const float *sx = g.tab, *sy = g.tab + g.NX, *sz = g.tab + g.NX + g.NY;
     const float sz0 = a0 ? __ldg(sz + z) : 0.f, sz1 = a0 ? __ldg(sz + min(z + 1, g.NZ - 1)) : 0.f;
     const float sy0 = a0 ? __ldg(sy + ya) : 0.f, sy1 = a1 ? __ldg(sy + ya + 1) : 0.f;
-    const float2 syz[2] = {make_float2(sy0 + sz0, sy0 + sz1), make_float2(sy1 + sz0, sy1 + sz1)};
+    // PAD: the three rates are added in acu_direct's order, x and y first
+    const float2 syz[2] = {PAD ? f2s(sy0) : make_float2(sy0 + sz0, sy0 + sz1),
+                           PAD ? f2s(sy1) : make_float2(sy1 + sz0, sy1 + sz1)};
+    const bool last = z + 1 >= g.NZ;                      // the second point is row padding
     const float hdt = 0.5f * g.dt;
     const float2 c0v = f2s(3.f * w.d2[0]), ih2 = f2s(g.ih * g.ih), one = f2s(1.f), two = f2s(2.f),
                  mone = f2s(-1.f);
@@ -1125,19 +1140,36 @@ acu_tma(GridDev g, FDW w, const float *u1, float *u0, float *__restrict__ grad,
 #pragma unroll
                 for (int r = 0; r < 2; r++) {
                     if (!ar[r]) continue;
-                    const float2 wv = lds2(I + L::WW * AIS + r * FZ), p0 = lds2(I + L::U0 * AIS + r * FZ);
-                    const float2 sd = f2mul(f2s(hdt), f2add(sxv, syz[r]));
-                    float2 num = f2mul(wv, lap[r]);
-                    num = f2fma(two, col[M + r], num);
-                    num = f2fma(f2add(sd, mone), p0, num);
-                    const float2 den = f2add(one, sd);
-                    const float2 un = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
+                    float2 wv = lds2(I + L::WW * AIS + r * FZ);      // w, or m
+                    const float2 p0 = lds2(I + L::U0 * AIS + r * FZ);
+                    float2 un;
+                    if constexpr (PAD) {
+                        if (last) wv.y = wv.x;
+                        const float2 d2 = f2s(g.dt * g.dt), sig = f2add(f2add(sxv, syz[r]), make_float2(sz0, sz1));
+                        const float2 A = f2mul(wv, f2fma(f2s(hdt), sig, one));
+                        const float2 nB = f2mul(wv, f2fma(f2s(hdt), sig, mone));
+                        const float2 num = f2fma(d2, lap[r], f2mul(f2add(wv, wv), col[M + r]));
+                        un = div_model(f2fma(nB, p0, num), A);
+                        if (last) un.y = 0.f;
+                    } else {
+                        const float2 sd = f2mul(f2s(hdt), f2add(sxv, syz[r]));
+                        float2 num = f2mul(wv, lap[r]);
+                        num = f2fma(two, col[M + r], num);
+                        num = f2fma(f2add(sd, mone), p0, num);
+                        const float2 den = f2add(one, sd);
+                        un = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
+                    }
                     const unsigned q = x * pl + qr[r];
                     st2(u0, q, un.x, un.y);
                     if (GRAD) {
                         const float2 uf = lds2(I + L::UF * AIS + r * FZ), gg = lds2(I + L::GG * AIS + r * FZ);
-                        const float2 t = f2fma(f2mul(mone, wv), uf, Z2);
-                        const float2 gn = f2fma(t, lap[r], gg);
+                        float2 gn;
+                        if constexpr (PAD) {
+                            gn = f2sub(gg, div_model(f2mul(f2mul(f2s(g.dt * g.dt), uf), lap[r]), wv));
+                        } else {
+                            const float2 t = f2fma(f2mul(mone, wv), uf, Z2);
+                            gn = f2fma(t, lap[r], gg);
+                        }
                         st2(grad, q, gn.x, gn.y);
                     }
                     if (check && !(isfinite(un.x) && isfinite(un.y))) atomicOr(flag, 1);
@@ -1442,7 +1474,7 @@ int tti_launch_any(prop_s *P, float *const *S, bool adjoint, const float *up, co
 
 // acoustic step: S[0] = u^n, S[1] = u^{n-1} (overwritten by u^{n+1});
 // grad != NULL: imaging with the forward field uf
-template <int M, int GRAD>
+template <int M, int GRAD, int PAD>
 int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
 {
     const GridDev &g = P->g;
@@ -1451,20 +1483,26 @@ int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
     using L = AL<M, GRAD>;
     AMaps am;
     bool ok = map_of(P, S[0], L::RC, L::RR, &am.u) && map_of(P, S[0], FZ, AFY, &am.q) &&
-              map_of(P, P->acw, FZ, AFY, &am.w) && map_of(P, S[1], FZ, AFY, &am.u0);
+              map_of(P, PAD ? P->m : P->acw, FZ, AFY, &am.w) && map_of(P, S[1], FZ, AFY, &am.u0);
     if (GRAD) ok = ok && map_of(P, uf, FZ, AFY, &am.uf) && map_of(P, grad, FZ, AFY, &am.g);
     if (!ok) return wp_fail(P, PROP_ECUDA, "cuTensorMapEncodeTiled failed");
     const size_t sb = M > 4 ? ring_bytes(AL<M, GRAD>::NS, AL<M, GRAD>::SZ)
                             : ring_smem(P, grd, 2, AL<M, GRAD>::SZ, AL<M, GRAD>::NS);
-    static const bool attr = set_smem(acu_tma<M, GRAD>, SMEM_MAX);
+    static const bool attr = set_smem(acu_tma<M, GRAD, PAD>, SMEM_MAX);
     (void)attr;
     const RecDev rec = GRAD ? RecDev{} : P->rec;
     grd.z += receiver_layers(rec, grd, blk);
-    launch_pass(acu_tma<M, GRAD>, grd, blk, sb, P->stream, g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am, P->flag,
-                                                  P->d.check_nan, rec, GRAD ? InjDev{} : P->inj, xc, P->flag);
+    launch_pass(acu_tma<M, GRAD, PAD>, grd, blk, sb, P->stream, g, P->w, S[0], P->out[0] ? P->out[0] : S[1], grad, am,
+                P->flag, P->d.check_nan, rec, GRAD ? InjDev{} : P->inj, xc, P->flag);
     P->kern_launches += 1;
     WP_CK(P, cudaGetLastError());
     return PROP_OK;
+}
+template <int M>
+int acu_launch(prop_s *P, float *const *S, const float *uf, float *grad)
+{
+    if (P->g.PZ != P->g.NZ) return grad ? acu_launch<M, 1, 1>(P, S, uf, grad) : acu_launch<M, 0, 1>(P, S, uf, grad);
+    return grad ? acu_launch<M, 1, 0>(P, S, uf, grad) : acu_launch<M, 0, 0>(P, S, uf, grad);
 }
 
 // Self-test of the bounded waits: one warp waits on an mbarrier that nothing
@@ -1545,10 +1583,10 @@ int acu_launch_tma(prop_s *P, float *const *S, const float *uf, float *grad)
     prof_begin(P, id);
     int rc;
     switch (P->M) {
-    case 2: rc = grad ? acu_launch<2, 1>(P, S, uf, grad) : acu_launch<2, 0>(P, S, uf, grad); break;
-    case 4: rc = grad ? acu_launch<4, 1>(P, S, uf, grad) : acu_launch<4, 0>(P, S, uf, grad); break;
-    case 6: rc = grad ? acu_launch<6, 1>(P, S, uf, grad) : acu_launch<6, 0>(P, S, uf, grad); break;
-    case 8: rc = grad ? acu_launch<8, 1>(P, S, uf, grad) : acu_launch<8, 0>(P, S, uf, grad); break;
+    case 2: rc = acu_launch<2>(P, S, uf, grad); break;
+    case 4: rc = acu_launch<4>(P, S, uf, grad); break;
+    case 6: rc = acu_launch<6>(P, S, uf, grad); break;
+    case 8: rc = acu_launch<8>(P, S, uf, grad); break;
     default: return wp_fail(P, PROP_EINVAL, "unsupported space order");
     }
     prof_end(P, id);
