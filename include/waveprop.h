@@ -37,10 +37,10 @@
  *   - Buffers may be host or device pointers (detected per pointer with
  *     cudaPointerGetAttributes).  The caller owns every buffer passed in or
  *     out; the library owns the handle and all device memory it allocates,
- *     and frees it in prop_destroy.  Freed memory, that of a call's buffers
- *     included, goes to a pool that the library's next allocations take it
- *     from: at most 1/16 of the device's memory, given back to the device
- *     when the last handle of the process is destroyed and by prop_trim.
+ *     and frees it in prop_destroy.  Memory freed meanwhile, that of a call's
+ *     buffers included, goes to a pool that the library's next allocations take
+ *     it from, while that pool holds no more than 1/16 of the device's memory in
+ *     all; prop_destroy and prop_trim give what is unused back to the device.
  *   - All work is enqueued on the stream given at prop_create (NULL = the
  *     legacy default stream); every call returns after that work completed.
  *   - Negative return = error.  After PROP_EINVAL the handle stays usable;

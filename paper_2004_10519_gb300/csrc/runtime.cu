@@ -47,11 +47,13 @@ int wp_cuda(prop_s *P, cudaError_t e, const char *what)
 // call (measured: 130 us for a small cudaMalloc + cudaFree, 0.6 ms per GB; an
 // acoustic gradient with 9.7 GB of stored levels spent 6 of its 32 ms on it, a
 // batch of eight small shots 13 of its 77).
-// The pool keeps at most 1/16 of the device's memory beyond what is in use; it
-// gives all of that back when the last handle of the process goes and on
-// prop_trim, and when an allocation does not fit (also one of the process
-// outside the library: the driver then takes unused pool memory back, checked
-// with a cudaMalloc of more than was free).  Its allocations and frees are
+// The pool lets go of unused memory, at its next synchronisation, while it holds
+// more than 1/16 of the device's memory, the used blocks included: so calls beside
+// handles and storage of more than that map and unmap theirs as cudaMalloc would.
+// It gives all that is unused back when a handle is destroyed and on prop_trim, and
+// when an allocation does not fit (also one of the process outside the library:
+// the driver then takes unused pool memory back, checked with a cudaMalloc of more
+// than was free).  Its allocations and frees are
 // ordered on a stream of its own, where each allocation is waited for and each
 // free comes after a synchronisation of the stream that used the block, so memory
 // passes between streams and threads as with cudaMalloc.  Not of the device: that
@@ -61,7 +63,6 @@ namespace {
 struct DevPool {
     cudaMemPool_t pool = nullptr;
     cudaStream_t st = nullptr;
-    int handles = 0;
 };
 constexpr int MAX_DEV = 64;
 DevPool g_pool[MAX_DEV];
@@ -142,19 +143,6 @@ static void dev_give_back(DevPool *d)
     if (!d) return;
     cudaStreamSynchronize(d->st);
     cudaMemPoolTrimTo(d->pool, 0);
-}
-// a handle of device `dev` was created (+1), not created after all (0) or destroyed (-1)
-static void count_handle(int dev, int n)
-{
-    DevPool *d = dev_pool(dev);
-    if (!d) return;
-    bool last;
-    {
-        std::lock_guard<std::mutex> lk(g_pool_mtx);
-        d->handles += n;
-        last = d->handles <= 0;
-    }
-    if (last) dev_give_back(d);
 }
 
 // All device allocations of the library go through here (prop_forward_noalloc
@@ -810,11 +798,10 @@ extern "C" int prop_create(const prop_desc *desc, const float *const *model, voi
         free_all(P);
         const int dev = P->dev;
         delete P;
-        count_handle(dev, 0);
+        dev_give_back(dev_pool(dev));
         tl_err = m;
         return rc;
     }
-    count_handle(P->dev, 1);
     *out = P;
     return PROP_OK;
 }
@@ -826,7 +813,7 @@ extern "C" void prop_destroy(prop_t *P)
     free_all(P);
     const int dev = P->dev;
     delete P;
-    count_handle(dev, -1);
+    dev_give_back(dev_pool(dev));
 }
 
 extern "C" const char *prop_last_error(const prop_t *P)

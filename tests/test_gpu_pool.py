@@ -65,3 +65,57 @@ def test_frees_beside_captures_of_another_thread(monkeypatch):
         for round_ in got[name]:
             for x, y in zip(round_, ref):
                 np.testing.assert_array_equal(x, y)
+
+
+def _free():
+    import torch
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _acoustic(wp, nt, n=192):
+    vp = np.full((n, n, n), 2.0, np.float32)
+    return wp.Propagator(wp.PROP_ACOUSTIC, (n, n, n), 4, 10.0, 4, nt, [vp], snap_mode=wp.SNAP_FULL_FP32)
+
+
+def _gradient(prop, nt):
+    wav = np.ones((1, nt), np.float32)
+    at = np.full((1, 3), 500.0, np.float32)
+    return prop.gradient(wav, at, at, np.zeros((1, nt), np.float32))[0]
+
+
+@pytest.mark.gpu
+def test_a_destroyed_handle_returns_its_memory_beside_others():
+    import paper_2004_10519_gb300 as wp
+    other, warm = _acoustic(wp, 4), _acoustic(wp, 4)
+    _gradient(warm, 4)
+    warm.close()
+    before = _free()
+    prop = _acoustic(wp, 40)                              # five fields of 32 MB, 39 levels in a gradient
+    _gradient(prop, 40)
+    assert before - _free() > 100 << 20
+    prop.close()
+    assert before - _free() < 8 << 20
+    other.close()
+
+
+@pytest.mark.gpu
+def test_allocation_takes_what_the_pool_holds_unused():
+    """A block larger than what the device has free and than any that the pool holds, but not than both."""
+    import torch
+    import paper_2004_10519_gb300 as wp
+    a, b = _acoustic(wp, 60), _acoustic(wp, 80)
+    _gradient(b, 80)                                      # modules, and what the answer is
+    ref = _gradient(b, 80)
+    b.trim()
+    full = _free()
+    _gradient(a, 60)
+    assert full - _free() > 1500 << 20                    # 59 levels of 32 MB, now unused
+    rest = torch.empty(_free() - (1 << 30), dtype=torch.uint8, device="cuda")
+    assert _free() < 1100 << 20
+    np.testing.assert_array_equal(_gradient(b, 80), ref)  # 79 levels
+    del rest
+    torch.cuda.empty_cache()
+    a.trim()
+    b.trim()
+    assert _free() > full - (300 << 20)                   # the work arrays went too; models stay
