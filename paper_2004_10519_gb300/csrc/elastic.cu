@@ -233,9 +233,14 @@ el_face2_kernel(GridDev g, Fields9 s, Fields9 xf0, Fields9 xf1, const float *__r
     const float2 a0 = ld(xf0.f[0], q), a1 = ld(xf0.f[1], q), a2 = ld(xf0.f[2], q);
     const float2 c0 = ld(xf1.f[0], q), c1 = ld(xf1.f[1], q), c2 = ld(xf1.f[2], q);
     // v^{k+1} - g v^k, the small difference of nearly equal values, in one fused
-    // operation; the quotient by g b_avg needs no more than its few last bits
+    // operation, and its quotient by g b_avg rounded from the rounded reciprocal (as
+    // div_by in tma.cuh): one division instead of two.  Elastic gradient, 200^3 so 8,
+    // forward and transposed step: two divisions 682 us, one 659, this 648, an
+    // approximate quotient 632; error of the b gradient against 64 bits, mean of 14
+    // models: 3.39e-7, 3.41e-7, 3.41e-7 and 3.45e-7
     auto face = [](float u, float v1, float v0, float gg, float b2) {
-        return u * __fdividef(__fmaf_rn(-gg, v0, v1), 0.5f * gg * b2);
+        const float n = __fmaf_rn(-gg, v0, v1), d = 0.5f * gg * b2, y = __frcp_rn(d), c = n * y;
+        return u * (isfinite(c) ? __fmaf_rn(__fmaf_rn(-d, c, n), y, c) : c);
     };
     st(f0, q, face(u0.x, c0.x, a0.x, gxh * gyn * gzn0, b0.x + bX.x), face(u0.y, c0.y, a0.y, gxh * gyn * gzn1, b0.y + bX.y));
     st(f1, q, face(u1.x, c1.x, a1.x, gxn * gyh * gzn0, b0.x + bY.x), face(u1.y, c1.y, a1.y, gxn * gyh * gzn1, b0.y + bY.y));
