@@ -903,7 +903,12 @@ WP_DEV void tti_upd_body(const GridDev &g, const FDW &w, const float *ex, const 
                 // remainder stays a normal number down to quotients of 2^-112
                 const float2 sc = f2s(4294967296.f), As = f2mul(A, sc);
                 const float2 yA = make_float2(__frcp_rn(As.x), __frcp_rn(As.y));
-                float2 pn = div_by(f2mul(f2fma(nB, p0, tp), sc), As, yA), rn = div_by(f2mul(f2fma(nB, r0, tr), sc), As, yA);
+                const float2 np = f2fma(nB, p0, tp), nr = f2fma(nB, r0, tr);
+                float2 pn = div_by(f2mul(np, sc), As, yA), rn = div_by(f2mul(nr, sc), As, yA);
+                if (!isfinite((pn.x + pn.y) + (rn.x + rn.y))) {      // infinite, NaN, or too large to be scaled
+                    pn = div_ieee(np, A);
+                    rn = div_ieee(nr, A);
+                }
                 if (!two) pn.y = rn.y = 0.f;
                 st2(pp, q, pn.x, pn.y);
                 st2(rp, q, rn.x, rn.y);
