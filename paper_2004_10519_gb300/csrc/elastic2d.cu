@@ -454,7 +454,7 @@ int launch_any(prop_s *P, float *const *S, float dt_sign)
 {
     const GridDev &g = P->g;
     const long long tiles = (long long)((g.NZ + QZ - 1) / QZ) * ((g.NX + 31) / 32);
-    return tiles >= 152 ? launch_tma<M, 32>(P, S, dt_sign) : launch_tma<M, 16>(P, S, dt_sign);
+    return tiles >= P->sms ? launch_tma<M, 32>(P, S, dt_sign) : launch_tma<M, 16>(P, S, dt_sign);
 }
 
 template <int M>

@@ -266,6 +266,7 @@ int run(prop_s *P, const prop_desc *d, const float *const *model, const float *w
         int dev = 0, sms = 152;
         WP_CK(P, cudaGetDevice(&dev));
         WP_CK(P, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        P->sms = sms;
         P->xchunk = stencil_xchunk(g, sms);
     }
     float *mdst[5] = {tti ? P->m : P->bu, tti ? P->c1 : P->lam, tti ? P->c2 : P->mu, P->th, P->ph};
