@@ -40,7 +40,8 @@
  *     and frees it in prop_destroy.  Memory freed meanwhile, that of a call's
  *     buffers included, goes to a pool that the library's next allocations take
  *     it from, while that pool holds no more than 1/16 of the device's memory in
- *     all; prop_destroy and prop_trim give what is unused back to the device.
+ *     all.  prop_destroy gives the device back what the handle held; prop_trim,
+ *     and the destruction of the last handle, all that is unused.
  *   - All work is enqueued on the stream given at prop_create (NULL = the
  *     legacy default stream); every call returns after that work completed.
  *   - Negative return = error.  After PROP_EINVAL the handle stays usable;

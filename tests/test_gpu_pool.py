@@ -90,12 +90,19 @@ def test_a_destroyed_handle_returns_its_memory_beside_others():
     other, warm = _acoustic(wp, 4), _acoustic(wp, 4)
     _gradient(warm, 4)
     warm.close()
+    other.trim()                                          # what the call's buffers left goes too
     before = _free()
-    prop = _acoustic(wp, 40)                              # five fields of 32 MB, 39 levels in a gradient
-    _gradient(prop, 40)
-    assert before - _free() > 100 << 20
+    prop = _acoustic(wp, 40)                              # model and state: four fields of 31 MB
+    assert before - _free() > 60 << 20
     prop.close()
     assert before - _free() < 8 << 20
+    prop = _acoustic(wp, 40)
+    _gradient(prop, 40)                                   # leaves the buffers of a call
+    held = _free()
+    prop.close()
+    assert _free() - held > 100 << 20                     # its own memory and the adjoint state's, at least
+    other.trim()
+    assert before - _free() < 8 << 20                     # and all that is unused
     other.close()
 
 
