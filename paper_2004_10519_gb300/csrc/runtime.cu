@@ -2366,11 +2366,14 @@ static bool lockstep_ok(prop_t *const *sh, int n)
             P->d.ckpt_interval != P0->d.ckpt_interval)
             return false;
     }
-    // the lockstep driver pays where the rounds are paced by the host (small
-    // windows: 32 windows of about 1 M points, 0.99 s against 1.01 s for
+    // the lockstep driver was chosen where the rounds are paced by the host
+    // (small windows: 32 windows of about 1 M points, 0.99 s against 1.01 s for
     // one thread per shot); on windows of tens of millions of points the
     // per-thread rendezvous measured 4 % faster (6.26 s against 6.51 s for 8
-    // shots of 30-110 M points).  WAVEPROP_LOCKSTEP=1 forces it, =0 disables it.
+    // shots of 30-110 M points).  Since a shot's own step has become two launches
+    // the small ones are no longer faster in lockstep: 0.91 s (TTI) and 1.54 s
+    // (elastic) against 0.86 and 1.53 s with the rendezvous, 0.84 and 1.41 s on
+    // launches of their own.  WAVEPROP_LOCKSTEP=1 forces it, =0 disables it.
     const char *e = getenv("WAVEPROP_LOCKSTEP");
     if (e && !strcmp(e, "0")) return false;
     if (e && !strcmp(e, "1")) return true;
@@ -2716,8 +2719,8 @@ static int gradient_lockstep(prop_t *const *shots, int n, const float *const *wa
 // checkpoint schedule, TMA-fed passes, checkpointed storage): as for TTI,
 // one host thread; the state and the adjoint state are updated in place, so
 // one fixed table serves every forward step and one per segment position
-// the transposed step with imaging (its three passes; the pointwise kernels
-// before and after it run per shot).  Full segments (K recomputed steps and
+// the transposed step with imaging (its three passes; the face products after
+// them run per shot).  Full segments (K recomputed steps and
 // K transposed steps) are captured once as a CUDA graph and replayed.
 // Each shot's operations are those of its own prop_gradient, in the same
 // order, so the results are the same bits.  Returns 1 (nothing done) if the

@@ -2358,8 +2358,8 @@ static int el_batch_run_fixed(TtiBatch *b, int slot, cudaStream_t st)
         el_vpass_batch<M, 0><<<nt, blk, sv, st>>>(D, b->dtiles, b->w);
         el_tpass_batch<M, 0><<<nt, blk, stt, st>>>(D, b->dtiles, b->w);
     } else {
-        // the three passes only: the pointwise kernels before and after are
-        // the caller's (per shot)
+        // the three passes only: the face products after them are the
+        // caller's (per shot)
         const size_t sv = ring_bytes(NSTAGE, VL<M>::SZ), s2 = ring_bytes(NSTAGE, TL<M, 2>::SZ),
                      s1 = ring_bytes(NSTAGE, TL<M, 1>::SZ);
         static const bool attr = set_smem(el_vpass_batch<M, 1>, sv) && set_smem(el_tpass_batch<M, 2>, s2) &&
